@@ -51,6 +51,15 @@ int dev_info(DevInfo *out) {
   return LAGP_OK;
 }
 
+int allow_smem(const void *fn, const DevInfo &di) {
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(di.smem_optin - fa.sharedSizeBytes));
+  return cuda_status(e);
+}
+
 // The unique id of the calling thread's current CUDA context (0 if it has none yet).  The
 // per-device caches of device addresses and constant uploads are keyed on it: after a
 // cudaDeviceReset the device's next context is a new one, whose constant banks are not
@@ -248,7 +257,7 @@ int lagp_check_take(int32_t *checked, int64_t *count, int32_t *site, int64_t *in
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_status(e);
   int (*const takes[])(CheckRec *) = {knn_check_take, select_check_take, select_mixed_check_take,
-                                      select_dense_check_take};
+                                      select_dense_check_take, predict_check_take};
   CheckRec first = {0ull, 0, 0, 0};
   unsigned long long total = 0ull;
   for (auto take : takes) {

@@ -27,7 +27,11 @@ __device__ __forceinline__ int tri_row(int e) {
 // dimension lda), carrying naug extra columns n .. n+naug-1 along so that they end as
 // L^{-1} b (forward substitution).  rl[k] receives 1 / l_kk.  Sets *fail (shared) on a
 // pivot <= 0; every thread returns after the same barriers.
-__device__ void chol_flat_fp64(double *A, int n, int lda, int naug, double *rl, int *fail) {
+// recip: the matrix entries (not the extra columns) are multiplied by 1 / l_kk instead of
+// divided by l_kk: the rounding of the FP64 recursion's candidate rows (select.cu), so a
+// design's rows come out bit for bit as that recursion forms them.
+__device__ void chol_flat_fp64(double *A, int n, int lda, int naug, double *rl, int *fail,
+                               bool recip = false) {
   const int tid = threadIdx.x, nt = blockDim.x;
   __syncthreads();
   if (tid == 0) {
@@ -44,7 +48,7 @@ __device__ void chol_flat_fp64(double *A, int n, int lda, int naug, double *rl, 
     for (int i = k + 1 + tid; i < n + naug; i += nt) {
       double *ap = (i < n) ? &A[i * lda + k] : &A[k * lda + i];
       const double a = *ap, q = a * r;
-      *ap = fma(fma(-q, lkk, a), r, q);
+      *ap = (recip && i < n) ? q : fma(fma(-q, lkk, a), r, q);
     }
     __syncthreads();
     // a_il -= l_ik l_lk for k < l <= i, and the extra columns: b_i -= l_ik b_k

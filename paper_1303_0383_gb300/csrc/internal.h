@@ -30,6 +30,10 @@ struct DevInfo {
   size_t smem_per_sm;
 };
 int dev_info(DevInfo *out);
+// Lets a kernel's launches use any dynamic shared memory the device allows.  The limit is state
+// of the function, not of a launch: setting each launch's own size would let one thread lower
+// it between another thread's setting and launch.
+int allow_smem(const void *fn, const DevInfo &di);
 
 // Kernel (a): candidate sets.
 size_t knn_workspace_bytes(int64_t N, int64_t T, int32_t ncand, int num_sms);
@@ -89,6 +93,13 @@ struct PredictArgs {
   double theta, g;
   const int32_t *idx;
   BatchView B;  // per-location tables, or designs == nullptr for a uniform launch
+  // the FP64 recursion's own rounding (chol_flat_fp64), and idx set to -1 where it fails
+  int32_t recip = 0;
+  // NN: the candidate lists (location t's M at its offset); the design, the n nearest, goes to
+  // idx where that is given
+  const int32_t *nn = nullptr;
+  int32_t M = 0;
+  int64_t N = INT64_MAX;
   double *mean, *s2, *var;
   int8_t *status;
 };
@@ -176,6 +187,7 @@ int knn_check_take(CheckRec *out);
 int select_check_take(CheckRec *out);
 int select_mixed_check_take(CheckRec *out);
 int select_dense_check_take(CheckRec *out);
+int predict_check_take(CheckRec *out);
 
 // Map the last CUDA error to a library code.
 int cuda_status(cudaError_t e);

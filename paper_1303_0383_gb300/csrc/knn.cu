@@ -609,8 +609,8 @@ int knn_launch_list(const double *X, int64_t N, int32_t p, const double *XX, int
     case 8: fn = (const void *)knn_kernel<8>; break;
     default: fn = (const void *)knn_kernel<0>; break;
   }
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  st = allow_smem(fn, di);
+  if (st) return st;
   int grid = knn_grid(nloc, di.num_sms, smem);
   if (ctas_per_sm > 0) {
     const int64_t g2 = (int64_t)di.num_sms * ctas_per_sm;
@@ -619,7 +619,7 @@ int knn_launch_list(const double *X, int64_t N, int32_t p, const double *XX, int
   char *w = static_cast<char *>(ws);
   unsigned int *bmax = reinterpret_cast<unsigned int *>(w);
   float *Xf = reinterpret_cast<float *>(w + 256);
-  e = cudaMemsetAsync(bmax, 0, sizeof(unsigned int), stream);
+  cudaError_t e = cudaMemsetAsync(bmax, 0, sizeof(unsigned int), stream);
   if (e != cudaSuccess) return cuda_status(e);
   const int64_t n = N * p;
   int pblocks = (int)((n + KB - 1) / KB);

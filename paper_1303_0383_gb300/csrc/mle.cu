@@ -365,9 +365,9 @@ int mle_launch(const MleArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream)
   if (ws_bytes < mle_workspace_bytes(a.T, a.n, di.num_sms)) return LAGP_ERR_INVALID_ARG;
   const bool sm = mle_in_smem(a.n);
   const size_t smem = sm ? mle_set_bytes(a.n) : 0;
-  cudaError_t e = cudaFuncSetAttribute(mle_fp64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  st = allow_smem(reinterpret_cast<const void *>(mle_fp64_kernel), di);
+  if (st) return st;
+  cudaError_t e;
   int G = mle_grid(a.T, a.n, di, sm);
   const int Gb = mle_grid_bound(a.T, di.num_sms);
   if (G > Gb) G = Gb;

@@ -31,6 +31,8 @@
 // live in shared memory.
 #include <math.h>
 
+#include <algorithm>
+
 #include "batch.cuh"
 #include "check.cuh"
 #include "fp64_exp.cuh"
@@ -282,12 +284,21 @@ size_t select_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, in
   if (method == LAGP_MSPE)
     return precision == LAGP_MIXED ? select_mspe_mixed_workspace_bytes(T, p, n, ncand, num_sms)
                                    : select_mspe_workspace_bytes(T, p, n, ncand, num_sms);
-  if (precision == LAGP_MIXED && method == LAGP_ALC)
-    return select_mixed_workspace_bytes(T, p, n, ncand, num_sms);
-  const size_t Mpad = (size_t)mpad_of(ncand);
-  const size_t G = (size_t)sel_grid(T, num_sms);
-  return 256 + align_up(G * (size_t)n * Mpad * sizeof(double), 256) +
-         align_up(G * (size_t)p * Mpad * sizeof(double), 256);
+  const size_t own = select_scratch_bytes_for_grid(sel_grid(T, num_sms), p, n, ncand);
+  if (method == LAGP_NN) return std::max(own, predict_fp64_workspace_bytes(T, n, num_sms));
+  return precision == LAGP_MIXED ? select_mixed_workspace_bytes(T, p, n, ncand, num_sms) : own;
+}
+
+// NN's design is given, so it is kernel (c) alone, on the n nearest candidates, with the
+// recursion's rounding (bit for bit this file's kernel).  GB300: 10000 locations at n = 50,
+// ncand = 1000, with the candidate search: 9.36 -> 2.00 ms; 3000 at n = 208: 27.5 -> 18.1 ms.
+static PredictArgs nn_args(const double *XX, int64_t T, int n, const int32_t *cand, int M, double *mean,
+                           double *s2, double *var, int32_t *idx, int8_t *status) {
+  PredictArgs pa;
+  pa.XX = XX; pa.T = T; pa.n = pa.nmax = n; pa.idx = idx;
+  pa.recip = 1; pa.nn = cand; pa.M = M;
+  pa.mean = mean; pa.s2 = s2; pa.var = var; pa.status = status;
+  return pa;
 }
 
 int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -302,35 +313,14 @@ int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t s
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  if (ws_bytes < select_workspace_bytes(a.T, a.p, a.n, a.M, a.method, a.precision, di.num_sms))
-    return LAGP_ERR_INVALID_ARG;
-  const int Mpad = mpad_of(a.M);
+  if (a.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(a.T, a.n, di.num_sms)) {
+    PredictArgs pa = nn_args(a.XX, a.T, a.n, a.cand, a.M, a.mean, a.s2, a.var, a.idx, a.status);
+    pa.X = a.X; pa.Z = a.Z; pa.p = a.p; pa.N = a.N; pa.theta = a.theta; pa.g = a.g;
+    pa.B = BatchView{nullptr, nullptr, nullptr, 0, a.theta_loc, nullptr};
+    return predict_fp64_launch(pa, ws, ws_bytes, stream);
+  }
   const int G = sel_grid(a.T, di.num_sms);
-  char *w = static_cast<char *>(ws);
-  SelParams P;
-  P.X = a.X; P.Z = a.Z; P.N = a.N; P.p = a.p; P.XX = a.XX; P.T = a.T; P.cand = a.cand;
-  P.M = a.M; P.Mpad = Mpad; P.n0 = a.n0; P.n = a.n; P.method = a.method;
-  P.theta = a.theta;
-  P.g = a.g;
-  P.nmax = a.n;
-  P.pmax = a.p;
-  P.B = BatchView{nullptr, nullptr, nullptr, 0, a.theta_loc, nullptr};
-  P.start = a.start; P.nstart = a.nstart;
-  P.r_min = a.r_min; P.n_out = a.n_out;
-  P.mean = a.mean; P.s2 = a.s2; P.var = a.var; P.idx = a.idx; P.status = a.status;
-  P.queue = reinterpret_cast<int *>(w);
-  P.U = reinterpret_cast<double *>(w + 256);
-  P.Xc = reinterpret_cast<double *>(w + 256 + align_up((size_t)G * a.n * Mpad * sizeof(double), 256));
-  const size_t smem = sel_smem_bytes(Mpad, a.n);
-  if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = cudaFuncSetAttribute(select_fp64_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
-  e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
-  if (e != cudaSuccess) return cuda_status(e);
-  select_fp64_kernel<<<G, SB, smem, stream>>>(P);
-  g_launches.fetch_add(1);
-  return cuda_status(cudaGetLastError());
+  return select_launch_on_grid(a, ws, ws_bytes, G, stream);
 }
 
 int select_default_grid(int64_t T, int num_sms) { return sel_grid(T, num_sms); }
@@ -369,9 +359,9 @@ int select_launch_on_grid(const SelectArgs &a, void *ws, size_t ws_bytes, int G,
   P.Xc = reinterpret_cast<double *>(w + 256 + align_up((size_t)G * a.n * Mpad * sizeof(double), 256));
   const size_t smem = sel_smem_bytes(Mpad, a.n);
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = cudaFuncSetAttribute(select_fp64_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  st = allow_smem(reinterpret_cast<const void *>(select_fp64_kernel), di);
+  if (st) return st;
+  cudaError_t e;
   e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);   // the work counter starts at zero
   if (e != cudaSuccess) return cuda_status(e);
   select_fp64_kernel<<<G, SB, smem, stream>>>(P);
@@ -398,8 +388,9 @@ size_t select_batch_workspace_bytes(const BatchLaunch &b, int num_sms) {
   if (b.method == LAGP_MSPE)
     return b.precision == LAGP_MIXED ? select_mspe_mixed_batch_workspace_bytes(b, G)
                                      : select_mspe_batch_workspace_bytes(b, G);
-  if (b.precision == LAGP_MIXED && b.method == LAGP_ALC) return select_mixed_batch_workspace_bytes(b, G);
-  return select_scratch_bytes_for_grid(G, b.pmax, b.nmax, b.Mmax);
+  const size_t own = select_scratch_bytes_for_grid(G, b.pmax, b.nmax, b.Mmax);
+  if (b.method == LAGP_NN) return std::max(own, predict_fp64_workspace_bytes(b.T, b.nmax, num_sms));
+  return b.precision == LAGP_MIXED ? select_mixed_batch_workspace_bytes(b, G) : own;
 }
 
 int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -415,6 +406,12 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
                                      : select_mspe_batch_launch(b, ws, ws_bytes, G, stream);
   if (b.precision == LAGP_MIXED && b.method == LAGP_ALC)
     return select_mixed_batch_launch(b, ws, ws_bytes, G, stream);
+  if (b.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms)) {
+    PredictArgs pa = nn_args(b.XX, b.T, b.nmax, b.cand, b.Mmax, b.mean, b.s2, b.var, b.idx, b.status);
+    pa.X = pa.Z = nullptr; pa.p = b.pmax; pa.theta = 1.0; pa.g = 0.0;
+    pa.B = BatchView{b.designs, b.locs, b.order, b.ldxx, nullptr, nullptr};
+    return predict_fp64_launch(pa, ws, ws_bytes, stream);
+  }
   if (ws_bytes < select_scratch_bytes_for_grid(G, b.pmax, b.nmax, b.Mmax)) return LAGP_ERR_INVALID_ARG;
   const int Mpad = mpad_of(b.Mmax);
   char *w = static_cast<char *>(ws);
@@ -431,9 +428,9 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
   P.Xc = reinterpret_cast<double *>(w + 256 + align_up((size_t)G * b.nmax * Mpad * sizeof(double), 256));
   const size_t smem = sel_smem_bytes(Mpad, b.nmax);
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = cudaFuncSetAttribute(select_fp64_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  st = allow_smem(reinterpret_cast<const void *>(select_fp64_kernel), di);
+  if (st) return st;
+  cudaError_t e;
   e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_status(e);
   select_fp64_kernel<<<G, SB, smem, stream>>>(P);
@@ -441,6 +438,9 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
   return cuda_status(cudaGetLastError());
 }
 
-int select_prepare() { return exp_table_upload(); }
+int select_prepare() {
+  const int st = exp_table_upload();
+  return st ? st : predict_fp64_prepare();
+}
 
 }  // namespace lagp

@@ -331,9 +331,9 @@ int select_dense_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
   o += L.idx;
   const size_t smem = dense_smem_bytes(Mpad, a.n);
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = cudaFuncSetAttribute(select_dense_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  st = allow_smem(reinterpret_cast<const void *>(select_dense_kernel), di);
+  if (st) return st;
+  cudaError_t e;
   e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_status(e);
   select_dense_kernel<<<G, DB, smem, stream>>>(P);

@@ -436,9 +436,9 @@ int mspe_run(MspeParams P, const MspeLayout &L, int G, char *w, int32_t *user_id
   off += L.idx;
   const size_t smem = mspe_smem_bytes(P.Mpad, P.nmax);
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = cudaFuncSetAttribute(select_mspe_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  const int st = allow_smem(reinterpret_cast<const void *>(select_mspe_kernel), di);
+  if (st) return st;
+  cudaError_t e;
   e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_status(e);
   select_mspe_kernel<<<G, TB, smem, stream>>>(P);

@@ -871,11 +871,10 @@ int mxm_run(MxParams P, const MxLayout &L, int G, char *w, int32_t *user_idx, co
   const bool ring = mxm_smem_bytes(P.Mpad, P.nmax, RING) <= di.smem_optin;
   const size_t smem = mxm_smem_bytes(P.Mpad, P.nmax, ring ? RING : 0);
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = ring ? cudaFuncSetAttribute(select_mspe_mixed_kernel<RING>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                       : cudaFuncSetAttribute(select_mspe_mixed_kernel<0>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+  const int st = allow_smem(ring ? reinterpret_cast<const void *>(select_mspe_mixed_kernel<RING>)
+                                 : reinterpret_cast<const void *>(select_mspe_mixed_kernel<0>), di);
+  if (st) return st;
+  cudaError_t e;
   e = cudaMemsetAsync(w, 0, 512, stream);  // work counter and re-score counter
   if (e != cudaSuccess) return cuda_status(e);
   if (ring)

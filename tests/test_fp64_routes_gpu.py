@@ -1,0 +1,52 @@
+"""NN by the predictive kernel alone against the FP64 recursion (which the no-allocation entry
+point runs on the same inputs): the predictive kernel makes the recursion's operations in its
+order, so designs, statuses and values must be the same bit for bit.  Sizes at the edges of
+the predictive kernel's group form (n = 208) and its teams (64 threads)."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from paper_1303_0383_gb300 import lagp
+
+pytestmark = pytest.mark.gpu
+
+
+def _both(N, p, T, n0, n, M, theta, g, method, seed):
+    import torch
+    rng = np.random.default_rng(seed)
+    X = rng.random((N, p))
+    Z = np.sin(3 * X[:, 0]) + X.sum(1)
+    XX = rng.random((T, p))
+    near = np.argsort(((XX[:, None] - X[None]) ** 2).sum(-1), axis=1, kind="stable")[:, :M]
+    d = lambda a: torch.as_tensor(np.ascontiguousarray(a)).cuda()
+    X, Z, XX, cand = d(X), d(Z), d(XX), d(near.astype(np.int32))
+    res = []
+    for call in ("workspace", "noalloc"):
+        o = dict(mean=torch.full((T,), 7.0, dtype=torch.float64, device="cuda"))
+        o["s2"], o["var"] = torch.full_like(o["mean"], 7.0), torch.full_like(o["mean"], 7.0)
+        o["idx"] = torch.full((T, n), -7, dtype=torch.int32, device="cuda")
+        o["status"] = torch.full((T,), 9, dtype=torch.int8, device="cuda")
+        a = (X, Z, XX, cand, n0, n, theta, g, method, "fp64", o["mean"], o["s2"], o["var"], o["idx"], o["status"])
+        if call == "workspace":
+            lagp.lagp_select_dev(*a, lagp.workspace(lagp.lagp_select_workspace_bytes(T, p, n, M, method)))
+        else:
+            code = lagp.lagp_select_dev_noalloc(*a)
+            assert code == lagp.LAGP_OK, lagp.strerror(code)
+        torch.cuda.synchronize()
+        res.append({k: v.cpu().numpy() for k, v in o.items()})
+    for k in res[0]:
+        assert np.array_equal(res[0][k], res[1][k], equal_nan=k not in ("idx", "status")), k
+    return res[0]
+
+
+@pytest.mark.parametrize("T,n,M", [(1, 3, 3), (700, 50, 60), (7, 64, 64), (310, 65, 70), (5, 208, 210),
+                                   (5, 209, 210), (2, 256, 256)])
+def test_nn_sizes(T, n, M):
+    r = _both(max(300, M), 2, T, 3, n, M, 0.1, 1e-4, "nn", T + n)
+    assert (r["status"] == 0).all()
+
+
+def test_nn_failed_factorisation():
+    r = _both(300, 2, 9, 3, 60, 60, 1e4, 0.0, "nn", 3)  # correlations of 1: no factor
+    assert (r["status"] != 0).any()
