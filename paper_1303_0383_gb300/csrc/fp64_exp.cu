@@ -41,6 +41,15 @@ void compute_host_consts(ExpConsts *c) {
   c->c2 = c2;
   c->c3 = c3;
   c->inv_ln2_64f = (float)(64.0L / ln2);
+  // fixed point (fx.cuh): 2^(-i/256) at 2^63, (ln2/256)^m / m! at 2^60
+  for (int i = 0; i < kFxTab; i++)
+    c->fx.tab[i] = (uint64_t)roundl(ldexpl(exp2l(-(long double)i / 256.0L), 63));
+  const long double a = ln2 / 256.0L;
+  c->fx.c1 = (uint64_t)roundl(ldexpl(a, 60));
+  c->fx.c2 = (uint64_t)roundl(ldexpl(a * a / 2.0L, 60));
+  c->fx.c3 = (uint32_t)roundl(ldexpl(a * a * a / 6.0L, 60));
+  c->fx.c4 = (uint32_t)roundl(ldexpl(a * a * a * a / 24.0L, 60));
+  c->fx.c5 = (uint32_t)roundl(ldexpl(a * a * a * a * a / 120.0L, 60));
 }
 
 __global__ void exp_eval_kernel(const double *__restrict__ x, double *__restrict__ y, int64_t n) {

@@ -18,6 +18,7 @@
 
 #include <mutex>
 
+#include "fx.cuh"
 #include "internal.h"
 
 namespace lagp {
@@ -31,6 +32,7 @@ struct ExpConsts {
   // significant bits (k * c1 exact for |k| < 2^13).
   float tabf_h[64], tabf_l[64];
   float c1, c2, c3, inv_ln2_64f;
+  FxConsts fx;  // the fixed-point version (fx.cuh)
 };
 
 // Host: the constants, computed once per process in long double (fp64_exp.cu).

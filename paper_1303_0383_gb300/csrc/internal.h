@@ -15,7 +15,6 @@ namespace lagp {
 constexpr int kMaxP = 8;
 constexpr int kMaxN = 256;       // local design size n
 constexpr int kMaxCand = 8192;   // candidate count
-#define LAGP_MIX_CTAS_PER_SM 3     // resident CTAs per SM of the mixed kernel
 
 extern std::atomic<int64_t> g_launches;
 
@@ -147,6 +146,7 @@ struct BatchLaunch {
   int32_t ldxx;
   const int32_t *cand;         // device; location t's list at locs[t].cand_off
   int32_t nmax, pmax, Mmax;
+  double gmin;                 // smallest nugget of the designs
   double *mean, *s2, *var;
   int32_t *idx;                // location t's indices at locs[t].idx_off
   int64_t idx_total;           // sum of the locations' n (the length of idx)
@@ -161,8 +161,8 @@ int select_mspe_prepare();
 int select_mspe_mixed_prepare();
 size_t select_batch_workspace_bytes(const BatchLaunch &b, int num_sms);
 int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream);
-size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b, int G);
-int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, int G, cudaStream_t stream);
+size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b);
+int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream);
 size_t select_mspe_batch_workspace_bytes(const BatchLaunch &b, int G);
 int select_mspe_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, int G, cudaStream_t stream);
 size_t select_mspe_mixed_batch_workspace_bytes(const BatchLaunch &b, int G);

@@ -371,7 +371,6 @@ int select_launch_on_grid(const SelectArgs &a, void *ws, size_t ws_bytes, int G,
 
 int select_max_ctas(int32_t method, int32_t precision) {
   if (method == LAGP_MSPE) return precision == LAGP_MIXED ? LAGP_MSPE_MIX_CTAS_PER_SM : 1;
-  if (precision == LAGP_MIXED && method == LAGP_ALC) return LAGP_MIX_CTAS_PER_SM;
   return 2;
 }
 
@@ -390,7 +389,7 @@ size_t select_batch_workspace_bytes(const BatchLaunch &b, int num_sms) {
                                      : select_mspe_batch_workspace_bytes(b, G);
   const size_t own = select_scratch_bytes_for_grid(G, b.pmax, b.nmax, b.Mmax);
   if (b.method == LAGP_NN) return std::max(own, predict_fp64_workspace_bytes(b.T, b.nmax, num_sms));
-  return b.precision == LAGP_MIXED ? select_mixed_batch_workspace_bytes(b, G) : own;
+  return b.precision == LAGP_MIXED ? select_mixed_batch_workspace_bytes(b) : own;
 }
 
 int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -405,7 +404,7 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
     return b.precision == LAGP_MIXED ? select_mspe_mixed_batch_launch(b, ws, ws_bytes, G, stream)
                                      : select_mspe_batch_launch(b, ws, ws_bytes, G, stream);
   if (b.precision == LAGP_MIXED && b.method == LAGP_ALC)
-    return select_mixed_batch_launch(b, ws, ws_bytes, G, stream);
+    return select_mixed_batch_launch(b, ws, ws_bytes, stream);
   if (b.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms)) {
     PredictArgs pa = nn_args(b.XX, b.T, b.nmax, b.cand, b.Mmax, b.mean, b.s2, b.var, b.idx, b.status);
     pa.X = pa.Z = nullptr; pa.p = b.pmax; pa.theta = 1.0; pa.g = 0.0;

@@ -1,45 +1,54 @@
-// select_mixed.cu -- kernels (b)+(c), mixed precision: float-float candidate screen on the
-// FP32 pipes, FP64 decisions and FP64 predictive equations.
+// select_mixed.cu -- kernels (b)+(c) for ALC: a candidate screen, FP64 decisions where it is
+// close, and FP64 predictive equations.
 //
 // Gramacy & Apley, Sec. 3: the greedy local design adds, at each step, the candidate that
 // maximises the ALC reduction cov_j(x,c)^2 / v_j(c) (Eq. dxy; SM Eq. dxy2).  The screen
 // carries, for every candidate, its row of the bordered Cholesky factor, v_j(c) and
-// cov_j(x,c) exactly as the FP64 kernel does (select.cu), but in float-float (FP32 pairs,
-// ff.cuh): on this GPU FP32 runs 58x faster than FP64, and plain FP32 cannot be used
-// because v_j(c) ~ g = 1e-6 is the difference of O(1) quantities.
+// cov_j(x,c) as the FP64 recursion does (select.cu).  FP64 runs at 1/64 of the FP32 rate on
+// this GPU, and plain FP32 cannot be used because v_j(c) ~ g = 1e-6 is the difference of O(1)
+// quantities, so there are two arithmetics (alc_screen.cuh): LAGP_MIXED screens in compensated
+// float-float on the FP32 pipe (46 bits), LAGP_FP64 in 64-bit fixed point on the integer pipe,
+// whose scores are as close to the exact ones as those of the FP64 recursion.
 //
 // Decisions stay FP64-exact where they are close: when the screen's second-best score is
 // within DELTA (relative) of its best, the design's FP64 Cholesky factor is rebuilt from
 // scratch and every candidate within DELTA is re-scored in FP64 (forward substitution,
 // one warp per candidate), the FP64 best winning with ties to the nearer candidate.
 // Otherwise the screen's best is taken.  DELTA = 1e-5 is about five times the largest
-// screen-vs-FP64 score discrepancy measured by emulation (2e-6 of the best score).
+// discrepancy between the FP64 scores and those of a screen of 46 bits, by emulation (2e-6
+// of the best score); with the fixed-point screen the factor and the re-score round exactly as
+// the FP64 recursion does, so that every decision is that recursion's.
 //
-// Each thread screens a pair of candidates with packed FP32 instructions (ff2.cuh), and a
-// step needs one block barrier: every thread merges the per-warp best/second-best results
-// and derives the step's pivot scalars itself.
+// Each thread screens a pair of candidates, and a step needs one block barrier: every thread
+// merges the per-warp best/second-best results and derives the step's pivot scalars itself.
+// The pivot's coordinates, state and factor row are read from a record that the warp holding
+// the step's best wrote before that barrier: no read of the row after it.
 //
-// The predictive equations (Eqs. predgp, preds2) are evaluated in FP64 on each selected
-// design with kernel (c)'s arithmetic (predict_loc.cuh) -- by this kernel itself right
-// after the design when the matrix fits in its shared memory, else by kernel (c) in
-// predict.cu afterwards -- so mu, s2 and V carry FP64 accuracy whatever precision
-// screened the candidates.
+// The predictive equations (Eqs. predgp, preds2) are evaluated in FP64 on the selected
+// designs by kernel (c) in predict.cu afterwards, so mu, s2 and V carry FP64 accuracy
+// whatever screened the candidates.
 #include <cooperative_groups.h>
 #include <math.h>
 #include <stdlib.h>
 
+#include "alc_screen.cuh"
 #include "batch.cuh"
 #include "check.cuh"
-#include "mixed_screen.cuh"
-#include "predict_loc.cuh"
 
 namespace lagp {
 namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int MB = 256;            // threads per CTA
 constexpr int kMaxCL = 8;          // CTAs per cluster in the cluster form
+constexpr int kScrThreads = 512;   // threads per SM: CTAs of 128, 256 or 512 threads, 128 registers each
+
+// A location's formats (fx.cuh), and what they are found from.
+struct FxFormat {
+  int fmt[2];           // sh2b, e
+  unsigned dmax, kmax;  // high words of the largest |x_c - x| and K(x, c)
+  int odd;              // a coordinate is not finite
+};
 
 struct MixParams {
   const double *X, *Z;
@@ -53,9 +62,9 @@ struct MixParams {
   double theta, theta_inv, g, onepg;
   BatchView B;     // per-location tables (B.designs == nullptr: uniform launch)
   int32_t *idx;   // selected design indices (required: the caller's or the workspace's)
-  float4 *U;     // slots of n x Qpad candidate pairs: row j of every candidate's factor row
-  int R;         // rows 0 .. R-1 live in shared memory instead
-  float4 *Xr;    // slots of p x Qpad pairs: candidate coordinates minus x
+  void *U;       // slots of n x Qpad candidate pairs: row j of every candidate's factor row
+  int smem;      // bytes of dynamic shared memory
+  void *Xr;      // slots of p x Qpad pairs: candidate coordinates minus x
   double *A;     // slots of n x (n + 2): FP64 factorisation
   int *queue;
   int *rescores; // count of FP64 re-score passes (diagnostics)
@@ -65,32 +74,104 @@ struct MixParams {
   int32_t *n_out;        // design sizes (T) when r_min > 1
   double *mean, *s2, *var;
   int8_t *status;
-  int fuse_pred;         // 1: the predictive equations here (matrix in shared memory)
   int CL;                // CTAs per cluster (cluster form): they share one location
-  int RT;                // tensor-memory instance: rows R .. R + RT - 1 also in tensor memory
+  int nrec;              // pivot records of a CTA
+  int tmem;              // 1: rows in tensor memory
 };
 
-#ifndef LAGP_MIX_MINB
-#define LAGP_MIX_MINB LAGP_MIX_CTAS_PER_SM  // 3 CTAs per SM, each with its first factor rows in shared memory
-#endif
-// The row-ring instances (one CTA per location) run up to 4 CTAs per SM: their rows come
-// from DRAM, and more warps in flight hide more of that (8-d workload, the shared-row-copy
-// instance at 4 CTAs per SM: 138.7 -> 133.1 ms).  At 4 CTAs per SM the instance without
-// the ring was slower (paper-2d 13.58 -> 15.25 ms: 3 rows in shared memory instead of 5).
-constexpr int kRingMinB = 4;
-__host__ __device__ constexpr int mix_minb(int RA, bool SR, bool CLU) {
-  (void)SR;
-  return (RA > 0 && !CLU) ? kRingMinB : LAGP_MIX_MINB;
+// FxArith: a location's state (one CTA): v = 1+g, cov_0(x, c) = K(x, c) in FP64, the coordinates
+// relative to x, in formats set by the largest coordinate difference and K(x, c) (compared by
+// the high words of their doubles, which are ordered like the values).  Returns whether every
+// step is to be decided in FP64: coordinates that are not finite, or spread so far that the
+// format's resolution, 2^(b-58), falls short of FP64's.
+template <int MBT>
+__device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, const double *etab, int4 *vp,
+                                         int4 *cp, int4 *Xr, unsigned char *used, int Qpad, FxFormat &F) {
+  const int tid = threadIdx.x, p = L.p, M = L.M;
+  long long *v = reinterpret_cast<long long *>(vp), *cov = reinterpret_cast<long long *>(cp);
+  // e even with 1 + g < 2^(e+1)
+  const int e = (ilogb(L.onepg) + 1) & ~1;
+  const long long onepg = __double2ll_rn(scalbn(L.onepg, 60 - e));
+  const double csc = sqrt(L.theta_inv * 1.4426950408889634);  // K = 2^-(squared distance) in these units
+  if (tid == 0) {
+    F.dmax = F.kmax = 0u;
+    F.odd = !(csc >= 0.0 && csc < INFINITY);
+  }
+  __syncthreads();
+  unsigned dmax = 0u, kmax = 0u;
+  for (int c = tid; c < 2 * Qpad; c += MBT) {
+    // (checked build: a design index past N gets v = 0, so that a start design holding it fails
+    // instead of reading its index)
+    const bool inside = c < M, live = inside && LAGP_CHK(L.cand[c], L.N, 24);
+    double kx = -1.0;  // no coordinates
+    if (live) {
+      const double *xc = L.X + (int64_t)L.cand[c] * p;
+      double acc = 0.0;
+      unsigned dm = 0u;
+      for (int k = 0; k < p; k++) {
+        const double dk = xc[k] - xl[k];
+        acc = fma(dk, dk, acc);
+        dm = max(dm, (unsigned)__double2hiint(dk) & 0x7fffffffu);
+      }
+      if (dm < 0x7ff00000u) {
+        kx = exp_nonpos(-acc * L.theta_inv, etab);
+        dmax = max(dmax, dm);
+        kmax = max(kmax, (unsigned)__double2hiint(kx) & 0x7fffffffu);
+      } else {
+        F.odd = 1;
+      }
+    }
+    used[c] = live ? 0 : 1;
+    v[c] = inside && !live ? 0 : onepg;
+    reinterpret_cast<double *>(cov)[c] = kx;
+  }
+  dmax = __reduce_max_sync(0xffffffffu, dmax);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if ((tid & 31) == 0) {
+    atomicMax(&F.dmax, dmax);
+    atomicMax(&F.kmax, kmax);
+  }
+  __syncthreads();
+  // coordinates at most 2^b in size; K(x, c) scaled by 2^(59 - e + w), the largest in
+  // [2^(59-e), 2^(60-e))
+  const int b = max(0, (int)(F.dmax >> 20) - 1023 + ilogb(csc) + 2);
+  const double fsc = scalbn(csc, 28 - b);
+  const int w = min(max(1023 - (int)(F.kmax >> 20), 0), 1022);
+  const double kw = scalbn(1.0, w), ke = scalbn(1.0, 59 - e);
+  for (int c = tid; c < 2 * Qpad; c += MBT) {
+    const double kx = reinterpret_cast<double *>(cov)[c];
+    const bool live = kx >= 0.0;
+    cov[c] = live ? __double2ll_rn(kx * kw * ke) : 0;
+    const double *xc = L.X + (live ? (int64_t)L.cand[c] * p : 0);
+    for (int k = 0; k < p; k++) {
+      const double f = live ? (xc[k] - xl[k]) * fsc : 0.0;
+      const int xh = __double2int_rn(f);
+      int *slot = reinterpret_cast<int *>(Xr + k * Qpad + (c >> 1)) + (c & 1);
+      slot[0] = xh;
+      slot[2] = __double2int_rn((f - (double)xh) * 1073741824.0);  // 2^30
+    }
+  }
+  if (tid == 0) {
+    F.fmt[0] = min(2 * b, 62);
+    F.fmt[1] = e;
+  }
+  return b > 8 || F.odd;
 }
-// RA: stages of the row ring (0: none).  SR: one shared copy of the step's factor row for
-// the whole CTA (one more block barrier per step) instead of one per warp, which frees
-// (MB/32 - 1) row copies of shared memory for the ring on large designs.
-// TM: rows R .. R + RT - 1 of each candidate are also kept in the CTA's tensor memory (128
-// columns: RT = 16, 8 or 4 rows for 1, 2 or up to 4 pairs per thread) and the screen reads
-// them from there instead of L2 (GB300, 24 warps per SM, four 16-byte loads per thread:
-// about 200 cycles from tensor memory against about 580 for L2 hits).  One CTA per location
-// only (not the cluster form); the ring instances run 4 CTAs per SM, which take all 512
-// columns, so the allocation never waits there either.
+
+// MBT threads per CTA, one location per CTA, one or two candidate pairs per thread up to 1024
+// candidates (more in turn beyond).  An SM always holds kScrThreads threads of 128 registers: a
+// spilled operand comes back from L2, since shared memory leaves no L1, and the row loops are
+// free of spills at 128 only.  A location of more candidates gets a larger share of an SM's
+// shared and tensor memory and fewer locations are in flight: the factor rows -- read again at
+// every later step -- then stay on the chip or in L2.  GB300, whole calls in float-float,
+// against three or four CTAs of 256 threads at 80 or 64 registers for every size, records of
+// the pivot gathered after the barrier and a ring of prefetched rows: 10000 2-d locations, n =
+// 50 of 1000, 14.05 -> 13.32 ms; 10000 8-d ones, n = 100 of 2000, 131.4 -> 118.2 ms; one location,
+// n = 50 of 1000, 524 -> 442 us.
+// TM: rows R .. R + RT - 1 of each candidate are also kept in the CTA's tensor memory (its
+// share of the 512 columns: 128 words per thread, RT = 32, 16 or 8 rows for 1, 2 or up to 4
+// pairs per thread) and the screen reads them from there instead of L2 (four 16-byte loads per
+// thread: about 200 cycles from tensor memory against about 580 for L2 hits).  One CTA per location only (not the cluster form).
 // CLU: the cluster form.  The P.CL CTAs of a thread-block cluster share one location, CTA
 // `crank` holding the candidate pairs crank*Qc .. crank*Qc + Qc - 1 (its own v, cov, flags,
 // factor rows and coordinates); a step's pivot state -- v_j(s), cov_j(x,s), u_s and x_s -- is
@@ -98,48 +179,36 @@ __host__ __device__ constexpr int mix_minb(int RA, bool SR, bool CLU) {
 // and the per-warp best scores are merged over the cluster after one cluster barrier.  With
 // 1/CL of the locations in flight, the live factor rows shrink by CL and more of each
 // CTA's rows fit in shared memory.  Every candidate's arithmetic is the same in both forms.
-template <int RA, bool SR, bool CLU, bool TM = false>
-__global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel(MixParams P) {
-  static_assert(!TM || !CLU, "tensor-memory rows: one CTA per location");
+template <class A, int MBT, int NP, bool CLU>
+__global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(const __grid_constant__ MixParams P) {
+  constexpr bool TM = !CLU;
+  using Word = typename A::Word;
+  constexpr int NWARP = MBT / 32;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int Qpad = P.Qpad, nmax = P.nmax;
-  constexpr int NW = SR ? 1 : MB / 32;                       // copies of the factor row
-  float4 *vp = reinterpret_cast<float4 *>(smraw);            // Qpad: v_j(c) pairs
-  float4 *cp = vp + Qpad;                                    // Qpad: cov_j(x, c) pairs
-  // copies of the new factor row: {h, h, -h, -h} and {l, l} per entry
-  const int nrow = (nmax + 1) & ~1;
-  float4 *wrow4 = reinterpret_cast<float4 *>(cp + Qpad);     // NW x nrow
-  float2 *wrow2 = reinterpret_cast<float2 *>(wrow4 + NW * nrow);  // NW x nrow
-  float2 *wxs = wrow2 + NW * nrow;                           // NW x kMaxP: new point
-  int *dr = reinterpret_cast<int *>(wxs + NW * kMaxP);       // nmax (padded to 4)
-  int *rlist = dr + ((nmax + 3) & ~3);                       // RESCORE_CAP
-  unsigned char *used = reinterpret_cast<unsigned char *>(rlist + RESCORE_CAP);  // Mpad
-  float4 *Us = reinterpret_cast<float4 *>(used + P.Mpad);    // R x Qpad: first factor rows
-  const int R = P.R;
-  float4 *ring = Us + (size_t)R * Qpad + threadIdx.x;        // RA x MB: row ring
-  // checked build: the layout above ends within the launch's dynamic shared memory
-  if (!LAGP_CHK(reinterpret_cast<unsigned char *>(Us + (size_t)R * Qpad + (size_t)RA * MB) - smraw,
-                dynamic_smem_bytes() + 1u, 20))
-    return;
-  __shared__ float tabh[64], tabl[64];
+  const int nmax = P.nmax;
+  __shared__ __align__(8) uint32_t ytab[A::kFixed ? 2 * kFxTab : 128];
   __shared__ double etab[64];
   __shared__ double xl[kMaxP];
-  constexpr int NRED = (MB / 32) * (CLU ? kMaxCL : 1);  // per-warp results (of the cluster)
-  __shared__ float red_s1[2][NRED], red_s2[2][NRED];
-  __shared__ int red_r1[2][NRED];
+  constexpr int NRED = NWARP * (CLU ? kMaxCL : 1);  // per-warp results (of the cluster)
+  __shared__ unsigned red_k1[2][NRED], red_k2[2][NRED];  // score keys, double-buffered by step
+  __shared__ int red_r1[2][NRED], red_buf[2][NWARP];
   __shared__ double xr_n[CLU ? kMaxCL : 1], xr_d[CLU ? kMaxCL : 1];  // per-CTA FP64 re-score bests
   __shared__ int xr_r[CLU ? kMaxCL : 1];
-  __shared__ double red_n[MB / 32], red_d[MB / 32];
-  __shared__ int red_rr[MB / 32];
+  __shared__ double red_n[NWARP], red_d[NWARP];
+  __shared__ int red_rr[NWARP];
   __shared__ int sh_loc, sh_fail, sh_nlist;
+  __shared__ LocParams L;  // the location's parameters: read where they are used
+  __shared__ FxFormat fx;                // the location's formats (FxArith)
+  __shared__ unsigned sh_top[3], sh_nwr[3];  // by step: best score key of the warps that are done,
+                                             // records begun
   __shared__ uint32_t sh_tmem;
   if constexpr (TM) {
-    // 128 columns of this SM's tensor memory (at most 3 CTAs per SM: 384 of 512, so the
-    // allocation never waits), released at the end of the kernel
+    // this CTA's share of the SM's tensor memory (the host checks that the resident CTAs'
+    // shares fit, so the allocation never waits), released at the end of the kernel
     if (threadIdx.x < 32) {
       asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                        (uint32_t)__cvta_generic_to_shared(&sh_tmem)),
-                   "n"(kTmemCols)
+                   "n"(tmem_cols(MBT))
                    : "memory");
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -147,25 +216,25 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   }
-  if (threadIdx.x < 64) {
-    tabh[threadIdx.x] = c_exp.tabf_h[threadIdx.x];
-    tabl[threadIdx.x] = c_exp.tabf_l[threadIdx.x];
-    etab[threadIdx.x] = c_exp.tab[threadIdx.x];
+  if (threadIdx.x < 64) etab[threadIdx.x] = c_exp.tab[threadIdx.x];
+  if constexpr (A::kFixed) {
+    for (int i = threadIdx.x; i < kFxTab; i += MBT)
+      reinterpret_cast<uint64_t *>(ytab)[i] = c_exp.fx.tab[i];
+  } else if (threadIdx.x < 64) {
+    ytab[threadIdx.x] = __float_as_uint(c_exp.tabf_h[threadIdx.x]);
+    ytab[64 + threadIdx.x] = __float_as_uint(c_exp.tabf_l[threadIdx.x]);
   }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int CL = CLU ? P.CL : 1;
   int crank = 0;
   if constexpr (CLU) crank = (int)cg::this_cluster().block_rank();
-  float4 *U = P.U + (size_t)blockIdx.x * nmax * Qpad;
-  float4 *Xr = P.Xr + (size_t)blockIdx.x * P.pmax * Qpad;
-  const int lda = nmax + 2;
-  double *A = P.A + (size_t)blockIdx.x * nmax * lda;
-  // this thread's tensor-memory words: its warp's lane quarter, its half of the columns
-  const uint32_t tb = TM ? sh_tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(64 * (warp >> 2))
+  Word *U = static_cast<Word *>(P.U) + (size_t)blockIdx.x * nmax * P.Qpad;
+  Word *Xr = static_cast<Word *>(P.Xr) + (size_t)blockIdx.x * P.pmax * P.Qpad;
+  const int lda = nmax + 1;
+  double *Af = P.A + (size_t)blockIdx.x * nmax * (nmax + 2);
+  // this thread's tensor-memory words: its warp's lane quarter, its part of the columns
+  const uint32_t tb = TM ? sh_tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)(kTmemWords * (warp >> 2))
                          : 0u;
-  float4 *srow4 = wrow4 + (SR ? 0 : warp) * nrow;  // this warp's copy of the new factor row
-  float2 *srow2 = wrow2 + (SR ? 0 : warp) * nrow;
-  float2 *sxs = wxs + (SR ? 0 : warp) * kMaxP;     // and of the new point's coordinates
 
   for (;;) {
     int qloc;  // the location's queue position (one per cluster in the cluster form)
@@ -181,14 +250,13 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
       qloc = sh_loc;
     }
     if (qloc >= P.T) break;
-    const LocParams L = resolve_loc(P.B, qloc, P.X, P.Z, P.XX, P.p, P.n, P.M, P.n0, P.theta,
-                                    P.g, P.cand, P.idx, P.N);
+    if (tid == 0)
+      L = resolve_loc(P.B, qloc, P.X, P.Z, P.XX, P.p, P.n, P.M, P.n0, P.theta, P.g, P.cand, P.idx, P.N);
+    __syncthreads();
     const int n = L.n, p = L.p, M = L.M;
     // checked build: the location fits the slot (rows, candidates, coordinates)
     if (!(LAGP_CHK(n - 1, nmax, 13) && LAGP_CHK(M - 1, CL * P.Mpad, 14) && LAGP_CHK(p - 1, P.pmax, 15)))
       continue;
-    const int32_t *cnd = L.cand;
-    const ff onepg = ff_from_double(L.onepg);
     // the start design: the n0 nearest, or a saved design (augmentation)
     const int n0e = P.start ? P.nstart : L.n0;
     // Without greedy steps (n0 == n) only the start design's own rows are ever read.
@@ -200,93 +268,131 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
     const int q0 = CLU ? crank * Qc : 0;
     const int Ql = CLU ? max(0, min(Qc, Qm - q0)) : Qm;
     const int Qs = CLU ? max(0, min(Ql, Q - q0)) : Q;
+    // Shared memory is laid out for the location: its pairs' v and cov, the pivot records, the
+    // design, the used flags, and as many of its factor rows as the rest holds.
+    const int Qpad = (Qc + 31) & ~31, nrow = (n + 1) & ~1, recw = A::rec_words(n);
+    Word *vp = reinterpret_cast<Word *>(smraw);                // Qpad: v_j(c) pairs
+    Word *cp = vp + Qpad;                                      // Qpad: cov_j(x, c) pairs
+    int2 *recs = reinterpret_cast<int2 *>(cp + Qpad);          // P.nrec x recw
+    int *dr = reinterpret_cast<int *>(recs + P.nrec * recw);   // n (padded to 4)
+    int *rlist = dr + ((n + 3) & ~3);                          // RESCORE_CAP
+    unsigned char *used = reinterpret_cast<unsigned char *>(rlist + RESCORE_CAP);  // 2 Qpad
+    Word *Us = reinterpret_cast<Word *>(used + 2 * Qpad);      // R x Qpad: first factor rows
+    int R = (P.smem - (int)(reinterpret_cast<unsigned char *>(Us) - smraw)) / (Qpad * (int)sizeof(Word));
+    R = R < n ? R & ~1 : n;  // even: every stretch of the row loops starts at an even entry
+    // rows R .. R + RT - 1 in tensor memory: 16, 8 or 4 rows per pair for up to 2, 4 or 8 pairs
+    // per thread (one: 32), so that they fit the thread's words in whole loads of four rows
+    const int slots = NP * ((Qpad + NP * MBT - 1) / (NP * MBT));
+    const int RT = TM && P.tmem ? 4 * (kTmemWords / 16 / slots) : 0;
+    // checked build: the layout above ends within the launch's dynamic shared memory
+    if (!LAGP_CHK(reinterpret_cast<unsigned char *>(Us + (size_t)R * Qpad) - smraw,
+                  dynamic_smem_bytes() + 1u, 20))
+      continue;
     if (tid < p) xl[tid] = L.x[tid];
     if (tid == 0) sh_fail = 0;
     __syncthreads();
-    // coordinates relative to x over sqrt(theta) (float-float pairs), v = 1+g,
-    // cov_0(x,c) = K(x,c) in FP64
-    for (int q = tid; q < Qpad; q += MB) {
-      ff cv[2];
-      bool flagged[2] = {false, false};  // checked build: a design index past N
-      for (int h = 0; h < 2; h++) {
-        const int c = 2 * q + h;             // this CTA's index
-        const int cgl = 2 * (q0 + q) + h;    // the location's candidate rank
-        bool live = CLU ? (q < Ql && cgl < M) : (c < M);
-        if (live && !LAGP_CHK(cnd[cgl], L.N, 11)) {
-          live = false;
-          flagged[h] = true;
-        }
-        cv[h] = ff{0.0f, 0.0f};
-        if (live) {
-          const double *xc = L.X + (int64_t)cnd[cgl] * p;
+    bool exact = false;  // (FxArith) every step is decided in FP64
+    if constexpr (A::kFixed) {
+      exact = fx_location<MBT>(L, xl, etab, vp, cp, Xr, used, Qpad, fx);
+    } else {
+      // coordinates relative to x over sqrt(theta), v = 1+g, cov_0(x,c) = K(x,c) in FP64, all as
+      // float-float pairs
+      const ff onepg = ff_from_double(L.onepg);
+      const double sc = sqrt(L.theta_inv);
+      for (int q = tid; q < Qpad; q += MBT) {
+        ff cv[2];
+        bool flagged[2] = {false, false};  // checked build: a design index past N
+        for (int h = 0; h < 2; h++) {
+          const int c = 2 * q + h;             // this CTA's index
+          const int cgl = 2 * (q0 + q) + h;    // the location's candidate rank
+          bool live = CLU ? (q < Ql && cgl < M) : (c < M);
+          if (live && !LAGP_CHK(L.cand[cgl], L.N, 11)) {
+            live = false;
+            flagged[h] = true;
+          }
+          cv[h] = ff{0.0f, 0.0f};
+          const double *xc = L.X + (live ? (int64_t)L.cand[cgl] * p : 0);
           double acc = 0.0;
-          const double sc = sqrt(L.theta_inv);  // the screen's coordinates are in units of sqrt(theta)
           for (int k = 0; k < p; k++) {
-            const double dk = xc[k] - xl[k];
+            const double dk = live ? xc[k] - xl[k] : 0.0;
             const ff fk = ff_from_double(dk * sc);
             float *slot = reinterpret_cast<float *>(Xr + k * Qpad + q);
             slot[h] = fk.h;
             slot[2 + h] = fk.l;
             acc = fma(dk, dk, acc);
           }
-          cv[h] = ff_from_double(exp_nonpos(-acc * L.theta_inv, etab));
-        } else {
-          for (int k = 0; k < p; k++) {
-            float *slot = reinterpret_cast<float *>(Xr + k * Qpad + q);
-            slot[h] = 0.0f;
-            slot[2 + h] = 0.0f;
-          }
+          if (live) cv[h] = ff_from_double(exp_nonpos(-acc * L.theta_inv, etab));
+          used[c] = live ? 0 : 1;
         }
-        used[c] = live ? 0 : 1;
+        // (a flagged candidate gets v = 0, so that a start design holding it fails instead of
+        // reading its index)
+        vp[q] = Word{(decltype(Word::x))(flagged[0] ? 0.0f : onepg.h), (decltype(Word::x))(flagged[1] ? 0.0f : onepg.h),
+                     (decltype(Word::x))(flagged[0] ? 0.0f : onepg.l), (decltype(Word::x))(flagged[1] ? 0.0f : onepg.l)};
+        cp[q] = Word{(decltype(Word::x))cv[0].h, (decltype(Word::x))cv[1].h, (decltype(Word::x))cv[0].l,
+                     (decltype(Word::x))cv[1].l};
       }
-      // (a flagged candidate gets v = 0, so that a start design holding it fails instead of
-      // reading its index)
-      vp[q] = make_float4(flagged[0] ? 0.0f : onepg.h, flagged[1] ? 0.0f : onepg.h,
-                          flagged[0] ? 0.0f : onepg.l, flagged[1] ? 0.0f : onepg.l);
-      cp[q] = make_float4(cv[0].h, cv[1].h, cv[0].l, cv[1].l);
     }
+    if (tid == 0) sh_top[0] = sh_nwr[0] = 0u;
     // Cluster form: the first steps read the start pivots' v, cov and coordinates from
     // the CTA holding them, so every CTA's state must be in place before any step begins
     // (a stale value read there would let the CTAs' decisions, and barriers, diverge).
     if constexpr (CLU) cg::this_cluster().sync();
     else __syncthreads();
-    if (P.start) start_ranks(P.start + L.loc * P.nstart, P.nstart, cnd, M, dr);
+    if (P.start) start_ranks(P.start + L.loc * P.nstart, P.nstart, L.cand, M, dr);
 
     int best = 0;
     int ne = n;       // the design's size (n, or where the stopping rule ends it)
-    ff vx = onepg;    // v_j(x), carried by every thread for the stopping rule
+    ff vx = ff_from_double(L.onepg);  // v_j(x), carried by every thread for the stopping rule
+    int csum = 0;     // (FxArith) cov has been shifted right by this much
+    // the pivot record in use, and whether it holds the step's pivot already
+    int active = 0;
+    bool have = false;
     for (int j = 0; j < n; j++) {
       const int s = (j < n0e) ? (P.start ? dr[j] : j) : best;
       if (s < 0) {  // nothing admissible left (the same for every thread)
         if (tid == 0) sh_fail = 1;
         break;
       }
-      // the pivot's CTA in the cluster (so) and its index there (sl), and that CTA's state
+      // the pivot's CTA in the cluster (so) and its index there (sl)
       int so = 0, sl = s;
-      const float4 *vps = vp, *cps = cp, *Uss = Us, *Ugs = U, *Xrs = Xr;
       if constexpr (CLU) {
         so = (s >> 1) / Qc;
         sl = s - 2 * so * Qc;
-        cg::cluster_group cl = cg::this_cluster();
-        vps = cl.map_shared_rank(vp, so);
-        cps = cl.map_shared_rank(cp, so);
-        Uss = cl.map_shared_rank(Us, so);
-        const size_t other = (size_t)((int)blockIdx.x - crank + so);
-        Ugs = P.U + other * nmax * Qpad;
-        Xrs = P.Xr + other * P.pmax * Qpad;
       }
-      const ff vs = ff2_get(vps, sl);
-      if (!(vs.h > 0.0f)) {
-        if (tid == 0) sh_fail = 1;
-        break;
+      if (CLU || !have) {
+        // a pivot whose record is not in place (forced, re-scored, or held by another CTA):
+        // every thread derives the scalars, the CTA gathers the row
+        const Word *vps = vp, *cps = cp, *Uss = Us, *Ugs = U, *Xrs = Xr;
+        if constexpr (CLU) {
+          cg::cluster_group cl = cg::this_cluster();
+          vps = cl.map_shared_rank(vp, so);
+          cps = cl.map_shared_rank(cp, so);
+          Uss = cl.map_shared_rank(Us, so);
+          const size_t other = (size_t)((int)blockIdx.x - crank + so);
+          Ugs = static_cast<const Word *>(P.U) + other * nmax * P.Qpad;
+          Xrs = static_cast<const Word *>(P.Xr) + other * P.pmax * P.Qpad;
+        }
+        if (!A::positive(vps, sl)) {
+          if (tid == 0) sh_fail = 1;
+          break;
+        }
+        const typename A::Scalars ps = A::scalars(vps, cps, sl);
+        active = 0;
+        int2 *rec = recs + active * recw;
+        for (int i = tid; i < j; i += MBT)
+          A::rec_entry(rec, i, nrow, (i < R ? Uss : Ugs) + (size_t)i * Qpad, sl);
+        if (tid < p) A::rec_coord(rec, tid, Xrs + tid * Qpad, sl);
+        if (tid == 0) A::scalars_store(rec, ps);
+        __syncthreads();
       }
-      // every thread derives the step's scalars itself: no barrier needed for them
-      const ff inv = ff_rcp(ff_sqrt(vs));
-      const ff uxj = ff_mul(ff2_get(cps, sl), inv);
-      if (P.r_min > 0.0) {
+      const int2 *rec = recs + active * recw;
+      if constexpr (A::kFixed) {
+        csum += A::scalars_load(rec).csh;
+      } else if (P.r_min > 0.0) {
         // Sec. 6 stopping rule: stop before a greedy point whose variance reduction ratio
         // v_j(x) / v_{j+1}(x) (psi cancels) is below r_min; every thread decides alike
-        const ff vxn = ff_sub(vx, ff_mul(uxj, uxj));
+        const ff ux = A::scalars_load(rec).ux;
+        const ff vxn = ff_sub(vx, ff_mul(ux, ux));
         if (j >= n0e && ff_to_double(vx) / ff_to_double(vxn) < P.r_min) {
           ne = j;
           break;
@@ -294,110 +400,111 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
         vx = vxn;
       }
       if (tid == 0) dr[j] = s;
-      if (crank == so && tid == ((sl >> 1) % MB)) used[sl] = 1;  // the pair's owner keeps the flags
-      // this warp's (or the CTA's) copy of the new factor row u_s and of x_s (relative to x)
-      {
-        const int i0 = SR ? tid : lane, st = SR ? MB : 32;
-        for (int i = i0; i < j; i += st) {
-          const ff u = ff2_get((i < R ? Uss : Ugs) + (size_t)i * Qpad, sl);
-          srow4[i] = make_float4(u.h, u.h, -u.h, -u.h);
-          srow2[i] = f2s(u.l);
-        }
-        if (i0 < p) {
-          const ff xk = ff2_get(Xrs + i0 * Qpad, sl);
-          sxs[i0] = make_float2(xk.h, xk.l);
-        }
-      }
-      if constexpr (SR) {
-        __syncthreads();
-      } else {
-        __syncwarp();
-      }
+      if (crank == so && tid == 0) used[sl] = 1;  // (the screen tests for the pivot itself)
       if (j == n - 1) break;
       const bool want = j + 1 >= n0e;
-      const ff2 inv2{f2s(inv.h), f2s(inv.l)}, uxj2{f2s(uxj.h), f2s(uxj.l)};
       float b1 = -1.0f, b2 = -1.0f;
       int r1 = 0x7fffffff;
-      const StepCtx C{U, Us, R, ring, Xr, vp, cp, srow4, srow2, sxs, tabh, tabl, inv2, uxj2,
-                      Qpad, p, j, 2 * q0, want, tb, TM ? P.RT : 0};
-      if constexpr (TM) {
-        // whole warps (tensor-memory accesses are warp-collective): pairs up to the next
-        // multiple of 32 (all within Qpad; those past Qs only update state nobody reads),
-        // a pair skipped only when the whole warp's are used
-        const int Q32 = (Qs + 31) & ~31;
-        for (int q = tid, ps = 0; q < Q32; q += MB, ps++) {
-          const bool u0 = used[2 * q], u1 = used[2 * q + 1];
-          if (__all_sync(0xffffffffu, u0 && u1)) continue;
-          screen_pair<RA, true>(C, q, u0, u1, b1, r1, b2, ps);
-        }
-      } else {
-        for (int q = tid; q < Qs; q += MB) {
-          const bool u0 = used[2 * q], u1 = used[2 * q + 1];
-          if (u0 && u1) continue;
-          screen_pair<RA>(C, q, u0, u1, b1, r1, b2);
-        }
+      const StepCtx<A> C{U, Us, R, Xr, vp, cp, used, rec, ytab, fx.fmt, Qpad, nrow, p, j,
+                         CLU && crank != so ? -1 : sl, 2 * q0, want, tb, RT};
+      // whole warps (tensor-memory accesses are warp-collective): pairs up to the next
+      // multiple of 32 (all within Qpad; those past Qs only update state nobody reads), each
+      // round's in two halves of whole warps
+      const int Q32 = (Qs + 31) & ~31;
+      for (int q = tid, k = 0; q - tid < Q32; q += NP * MBT, k += NP) {
+        const int left = Q32 - (q - tid), dq = NP == 1 ? MBT : min(MBT, ((left >> 1) + 31) & ~31);
+        if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, q, b1, r1, b2, k, q + dq < Q32 ? dq : 0);
       }
-      // best and second-best screen scores: warp shuffles, one barrier, then every
-      // thread merges the per-warp results itself (double-buffered by step parity)
+      // best and second-best screen scores of the warp; the warp writes the record of its own
+      // best candidate as the next step's pivot before the barrier, so that the gather of the
+      // row (L2) and the scalars are off the path between the barrier and the next screen.
+      // Only a warp ahead of all that are done writes one (the winner always is; of eight warps
+      // in any order, 2.7 on average), in the records other than the one in use in turn; where
+      // they run out, the CTA gathers the pivot after the barrier.
       const int par = j & 1;
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ob1 = __shfl_down_sync(0xffffffffu, b1, o);
-        const float ob2 = __shfl_down_sync(0xffffffffu, b2, o);
-        const int orr = __shfl_down_sync(0xffffffffu, r1, o);
-        merge2(ob1, orr, ob2, b1, r1, b2);
-      }
-      if (lane == 0) {
-        if constexpr (CLU) {  // into every CTA of the cluster
-          cg::cluster_group cl = cg::this_cluster();
-          const int e = crank * (MB / 32) + warp;
-          for (int r = 0; r < CL; r++) {
-            cl.map_shared_rank(&red_s1[par][0], r)[e] = b1;
-            cl.map_shared_rank(&red_s2[par][0], r)[e] = b2;
-            cl.map_shared_rank(&red_r1[par][0], r)[e] = r1;
+      if (tid == 0) sh_top[(j + 1) % 3] = sh_nwr[(j + 1) % 3] = 0u;  // (last used two steps ago)
+      if (want) {
+        unsigned k1 = score_key(b1), k2 = score_key(b2);
+        warp_best2(k1, r1, k2);
+        unsigned top = 0u;
+        if (!CLU && lane == 0) top = atomicMax(&sh_top[j % 3], k1);
+        int buf = -1;
+        if (!CLU && k1 && k1 >= __shfl_sync(0xffffffffu, top, 0)) {
+          if (lane == 0) buf = (int)atomicAdd(&sh_nwr[j % 3], 1u);
+          buf = __shfl_sync(0xffffffffu, buf, 0);
+          buf = buf < P.nrec - 1 ? buf + (buf >= active ? 1 : 0) : -1;
+        }
+        if (buf >= 0) {
+          const int sl2 = r1;
+          int2 *nrec_ = recs + buf * recw;
+          __syncwarp();  // this step's rows, v and cov of the warp's candidates are in place
+          if (j + 2 < n)
+            for (int i = lane; i <= j; i += 32)
+              A::rec_entry(nrec_, i, nrow, (i < R ? Us : U) + (size_t)i * Qpad, sl2);
+          if (lane < p) A::rec_coord(nrec_, lane, Xr + lane * Qpad, sl2);
+          const typename A::Scalars np = A::scalars(vp, cp, sl2);
+          if (lane == 0) A::scalars_store(nrec_, np);
+        }
+        if (lane == 0) {
+          if constexpr (CLU) {  // into every CTA of the cluster
+            cg::cluster_group cl = cg::this_cluster();
+            const int en = crank * NWARP + warp;
+            for (int r = 0; r < CL; r++) {
+              cl.map_shared_rank(&red_k1[par][0], r)[en] = k1;
+              cl.map_shared_rank(&red_k2[par][0], r)[en] = k2;
+              cl.map_shared_rank(&red_r1[par][0], r)[en] = r1;
+            }
+          } else {
+            red_k1[par][warp] = k1;
+            red_k2[par][warp] = k2;
+            red_r1[par][warp] = r1;
+            red_buf[par][warp] = buf;
           }
-        } else {
-          red_s1[par][warp] = b1;
-          red_s2[par][warp] = b2;
-          red_r1[par][warp] = r1;
         }
       }
       if constexpr (CLU) cg::this_cluster().sync();
       else __syncthreads();
+      have = false;
       if (!want) continue;
-      float B1 = red_s1[par][0], B2 = red_s2[par][0];
-      int R1 = red_r1[par][0];
-      if constexpr (CLU) {
-        // the cluster's 8 CL entries: lane l merges entries l and l + 32, then a butterfly
-        // over the warp (the merge is order-independent: a unique best, ties to the smaller
-        // rank, and the largest other score)
-        const int ne = CL * (MB / 32);
-        B1 = -1.0f;
-        B2 = -1.0f;
-        R1 = 0x7fffffff;
-        for (int w = lane; w < ne; w += 32) merge2(red_s1[par][w], red_r1[par][w], red_s2[par][w], B1, R1, B2);
-        for (int o = 16; o > 0; o >>= 1) {
-          const float ob1 = __shfl_xor_sync(0xffffffffu, B1, o);
-          const float ob2 = __shfl_xor_sync(0xffffffffu, B2, o);
-          const int orr = __shfl_xor_sync(0xffffffffu, R1, o);
-          merge2(ob1, orr, ob2, B1, R1, B2);
-        }
-      } else {
-        for (int w = 1; w < MB / 32; w++)
-          merge2(red_s1[par][w], red_r1[par][w], red_s2[par][w], B1, R1, B2);
+      // every warp merges the CTA's (the cluster's) entries: lane l takes entries l, l + 32
+      unsigned K1 = 0u, K2 = 0u;
+      int R1 = 0x7fffffff;
+      const int nred = CL * NWARP;
+      if (lane < nred) {
+        K1 = red_k1[par][lane];
+        K2 = red_k2[par][lane];
+        R1 = red_r1[par][lane];
       }
-      best = (R1 == 0x7fffffff) ? -1 : R1;
-      const bool near = R1 != 0x7fffffff && B2 >= B1 * (1.0f - DELTA);
+      if (CLU && lane + 32 < nred) merge_keys(red_k1[par][lane + 32], red_r1[par][lane + 32],
+                                              red_k2[par][lane + 32], K1, R1, K2);
+      const int ew = warp_best2(K1, R1, K2);
+      best = K1 ? R1 : -1;
+      if (!CLU && K1) {
+        const int buf = red_buf[par][ew];
+        have = buf >= 0;
+        if (have) active = buf;
+      }
+      // Candidates closer than DELTA are decided in FP64.  For the FP64 precision the margin
+      // also covers the FP64 recursion's own rounding of cov_j(x, c) where that is small
+      // (2^-46 of the largest K(x, c)).
+      float delta = DELTA;
+      if constexpr (A::kFixed) {
+        if (K1) delta += scalbnf(1.0f, 13 - csum) / fmaxf(fabsf(fx_to_float(A::get64(cp, best))), 1.0f);
+        if (exact) delta = 1.0f;
+      }
+      const float B1 = __uint_as_float(K1 - 1u), B2 = __uint_as_float(K2 - 1u);
+      const bool near = K1 && ((K2 && B2 >= B1 * (1.0f - delta)) || exact);
       if (!near) continue;
       // ---- FP64 re-score of the near-tied candidates (rare) ----
       if (tid == 0 && crank == 0 && P.rescores) atomicAdd(P.rescores, 1);
       // each CTA re-scores its own near-tied candidates (the FP64 factor of the design, the
       // same in every CTA, is formed by each)
-      const RescoreCtx R{L.X, cnd, xl, etab, used, vp, cp, dr, A, rlist, &sh_nlist, &sh_fail,
+      const RescoreCtx R{L.X, L.cand, xl, etab, used, vp, cp, dr, Af, Af + nmax * lda, rlist, &sh_nlist, &sh_fail,
                          red_n, red_d, red_rr, p, 2 * q0, CLU ? min(2 * Ql, M - 2 * q0) : M, j + 1, lda,
-                         L.theta_inv, L.onepg};
+                         L.theta_inv, L.onepg, delta, A::kFixed};
       double bn, bd;
       int br;
-      rescore_fp64(R, B1, &bn, &bd, &br);
+      rescore_fp64<A>(R, B1, &bn, &bd, &br);
       if (sh_fail) break;  // the same in every CTA of a cluster
       if constexpr (CLU) {  // the cluster's FP64 best, ties to the nearer candidate
         cg::cluster_group cl = cg::this_cluster();
@@ -418,7 +525,9 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
             br = xr_r[r];
           }
       }
-      best = (br != 0x7fffffff) ? br : best;
+      const int rb = br != 0x7fffffff ? br : A::kFixed ? -1 : best;
+      if (rb != best) have = false;
+      best = rb;
     }
     // (cluster form: the last step's pivot reads of the other CTAs' state are done before
     // any CTA moves on and reuses or discards it)
@@ -427,29 +536,16 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
     // the design (design indices), or -1 when a step failed; kernel (c) (predict.cu)
     // evaluates the predictive equations on it in FP64
     if (crank == 0) {
-      for (int i = tid; i < n; i += MB) L.idx[i] = (sh_fail || i >= ne) ? -1 : cnd[dr[i]];
+      for (int i = tid; i < n; i += MBT)
+        L.idx[i] = (sh_fail || i >= ne || !LAGP_CHK(dr[i], M, 16)) ? -1 : L.cand[dr[i]];
       if (P.n_out && tid == 0) P.n_out[L.loc] = sh_fail ? 0 : ne;
-    }
-    // The predictive equations on the design (kernel (c)'s arithmetic, predict_loc.cuh),
-    // here while the other resident CTAs screen -- FP64 work beside their FP32 work -- when
-    // the matrix fits in the shared-memory factor rows (dead now); the reciprocal pivots go
-    // to the per-warp row copies.  Otherwise kernel (c) runs after this kernel.  Only
-    // the instance without the row ring carries this code (in the other it costs 2 % on
-    // the 8-d workload, which has no room for the matrix anyway).
-    if constexpr (RA == 0 && !CLU) {
-      if (P.fuse_pred) {
-        __syncthreads();  // every thread reads the design below
-        predict_location(L, L.idx, sh_fail ? n : ne, xl, reinterpret_cast<double *>(Us),
-                         reinterpret_cast<double *>(wrow4), etab, &sh_fail, L.loc, P.mean, P.s2,
-                         P.var, P.status);
-      }
     }
     // The factor rows in global memory are dead now (the next location rewrites each row
     // before reading it): drop their L2 lines without writing them back to DRAM.
     {
       char *u0 = reinterpret_cast<char *>(U + (size_t)R * Qpad);
-      const int nlines = (int)(((size_t)(n > R ? n - R : 0) * Qpad * sizeof(float4)) / 128);
-      for (int l = tid; l < nlines; l += MB)
+      const int nlines = (int)(((size_t)(n > R ? n - R : 0) * Qpad * sizeof(int4)) / 128);
+      for (int l = tid; l < nlines; l += MBT)
         asm volatile("discard.global.L2 [%0], 128;" ::"l"(u0 + (size_t)l * 128) : "memory");
     }
   }
@@ -461,7 +557,7 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (threadIdx.x < 32)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(sh_tmem),
-                   "n"(kTmemCols)
+                   "n"(tmem_cols(MBT))
                    : "memory");
   }
 }
@@ -470,38 +566,36 @@ __global__ void __launch_bounds__(MB, mix_minb(RA, SR, CLU)) select_mixed_kernel
 // shared-memory rows after the Mpad = 2 Qpad flag bytes start 16-byte aligned).
 int mix_qpad(int M, int CL) { return (int)align_up((size_t)ceil_div(ceil_div(M, 2), CL), 32); }
 
-// Dynamic shared memory: the per-candidate state, then the first R factor rows and the
-// threads' row rings (RA stages).
-size_t mix_smem_bytes(int Qpad, int n, int R, int RA, bool SR) {
-  const size_t nrow = (size_t)((n + 1) & ~1);
-  const size_t nw = SR ? 1 : MB / 32;
-  return (size_t)Qpad * 2 * sizeof(float4) +
-         nw * (nrow * (sizeof(float4) + sizeof(float2)) + kMaxP * sizeof(float2)) +
-         (size_t)((n + 3) & ~3) * sizeof(int) + RESCORE_CAP * sizeof(int) + (size_t)2 * Qpad +
-         (size_t)R * Qpad * sizeof(float4) + (size_t)RA * MB * sizeof(float4);
-}
-
-// The kernel instance of a launch: ring stages RA (0 or RING_A), a shared factor-row copy
-// SR, and CL CTAs per location (CL > 1: the cluster form).
+// The kernel instance of a launch: threads per CTA and CTAs per location (CL > 1: the cluster
+// form, 256 threads).
 struct MixVariant {
-  int RA;
-  bool SR;
+  int MBT;
+  int NP;      // pairs a thread takes at a time
   int CL;
-  bool TM = false;  // rows R .. R + RT - 1 also in tensor memory (RA == 0, CL == 1)
+  bool fixed;  // FxArith (LAGP_FP64) instead of FfArith (LAGP_MIXED)
 };
 
+// Pivot records of a CTA: the one in use and up to six begun in a step; fewer where the rest of
+// the state would leave the SM fewer CTAs.
+constexpr int kRecords = 7;
+
+// Dynamic shared memory without the factor rows.
+size_t mix_state_bytes(int Qpad, int n, int nrec, MixVariant v) {
+  const size_t recw = v.fixed ? FxArith::rec_words(n) : FfArith::rec_words(n);
+  return (size_t)Qpad * 2 * sizeof(int4) + nrec * recw * sizeof(int2) +
+         (size_t)((n + 3) & ~3) * sizeof(int) + RESCORE_CAP * sizeof(int) + (size_t)2 * Qpad;
+}
+
+template <class A>
+const void *mix_kernel_of(int MBT, int NP) {
+  return NP == 1      ? reinterpret_cast<const void *>(select_mixed_kernel<A, 128, 1, false>)
+         : MBT == 128 ? reinterpret_cast<const void *>(select_mixed_kernel<A, 128, 2, false>)
+         : MBT == 256 ? reinterpret_cast<const void *>(select_mixed_kernel<A, 256, 2, false>)
+                      : reinterpret_cast<const void *>(select_mixed_kernel<A, 512, 2, false>);
+}
 const void *mix_kernel(MixVariant v) {
-  if (v.CL > 1)
-    return v.RA ? reinterpret_cast<const void *>(select_mixed_kernel<RING_A, false, true>)
-                : reinterpret_cast<const void *>(select_mixed_kernel<0, false, true>);
-  if (!v.RA)
-    return v.TM ? reinterpret_cast<const void *>(select_mixed_kernel<0, false, false, true>)
-                : reinterpret_cast<const void *>(select_mixed_kernel<0, false, false>);
-  if (v.SR)
-    return v.TM ? reinterpret_cast<const void *>(select_mixed_kernel<RING_A, true, false, true>)
-                : reinterpret_cast<const void *>(select_mixed_kernel<RING_A, true, false>);
-  return v.TM ? reinterpret_cast<const void *>(select_mixed_kernel<RING_A, false, false, true>)
-              : reinterpret_cast<const void *>(select_mixed_kernel<RING_A, false, false>);
+  if (v.CL > 1) return reinterpret_cast<const void *>(select_mixed_kernel<FfArith, 256, 2, true>);
+  return v.fixed ? mix_kernel_of<FxArith>(v.MBT, v.NP) : mix_kernel_of<FfArith>(v.MBT, v.NP);
 }
 
 size_t mix_static_smem(MixVariant v) {
@@ -509,67 +603,44 @@ size_t mix_static_smem(MixVariant v) {
   return cudaFuncGetAttributes(&fa, mix_kernel(v)) == cudaSuccess ? fa.sharedSizeBytes : 4096;
 }
 
-int mix_minb(MixVariant v) { return mix_minb(v.RA, v.SR, v.CL > 1); }
-
-size_t mix_resident(int Qpad, int n, MixVariant v, const DevInfo &di) {
-  const size_t per = mix_static_smem(v) + 1024 + mix_smem_bytes(Qpad, n, 0, v.RA, v.SR);
-  const size_t k = di.smem_per_sm / per;  // 1 KB reserved per CTA
-  const size_t mb = (size_t)mix_minb(v);
-  return k < mb ? k : mb;
-}
+// Resident CTAs per SM the instance is compiled for.
+int mix_minb(MixVariant v) { return kScrThreads / v.MBT; }
 
 // Launch-shape overrides for measurements (they change no result): LAGP_MIX_CLUSTER = CTAs
-// per location (1, 2, 4 or 8), LAGP_MIX_RING = 0 / 1 (row ring off / on).  -1: not set.
+// per location (1, 2, 4 or 8), LAGP_MIX_TMEM = 0 (no rows in tensor memory).  -1: not set.
 int mix_env(const char *name) {
   const char *e = getenv(name);
   return e && *e ? atoi(e) : -1;
 }
 
-// CTAs per location: the cluster form where a location's factor rows are large enough that
-// the rows of all locations in flight overflow L2.
-int mix_cluster_size(int n, int M) {
+// One CTA per location: the cluster form (several) measured slower on every workload.
+int mix_cluster_size() {
   const int e = mix_env("LAGP_MIX_CLUSTER");
-  if (e == 1 || e == 2 || e == 4 || e == 8) return e;
-  (void)n;
-  (void)M;
-  return 1;
+  return e == 1 || e == 2 || e == 4 || e == 8 ? e : 1;
 }
 
-// The row ring is used where a CTA's factor rows (n x M float-float entries) come mostly
-// from DRAM -- 8-d workload (n = 100, M = 2000) yes, paper-2d (n = 50, M = 1000) no, both
-// measured -- and only if its shared memory leaves at least as many CTAs resident per SM;
-// with one shared copy of the factor row where the per-warp copies are what leave no room
-// (the 8-d workload at 4 CTAs per SM, the batched workload's large n).  The cluster form has
-// no shared-copy instance.
-MixVariant mix_variant(int n, int M, int CL, const DevInfo &di) {
-  const int Qpad = mix_qpad(M, CL);
-  const MixVariant plain{0, false, CL}, ring{RING_A, false, CL}, ring_sr{RING_A, true, CL};
-  const int er = mix_env("LAGP_MIX_RING");
-  if (er == 0) return plain;
-  if (er == 1) return ring;
-  if ((int64_t)n * M < 100000 * (int64_t)CL) return plain;
-  // the most resident CTAs per SM wins; at a tie, the ring with per-warp row copies (no
-  // extra barrier per step)
-  const size_t k0 = mix_resident(Qpad, n, plain, di);
-  const size_t kr = mix_resident(Qpad, n, ring, di);
-  const size_t ks = CL == 1 ? mix_resident(Qpad, n, ring_sr, di) : 0;
-  if (kr >= k0 && kr >= ks) return ring;
-  if (ks >= k0) return ring_sr;
-  return plain;
+// Threads per CTA: one candidate pair per thread where 256, 512 or 1024 threads cover them.
+MixVariant mix_variant(int M, int CL, bool fixed) {
+  if (CL > 1) return MixVariant{256, 2, CL, false};
+  const int Qpad = mix_qpad(M, 1);
+    return MixVariant{Qpad <= 256 ? 128 : Qpad <= 512 ? 256 : 512, Qpad <= 128 ? 1 : 2, 1, fixed};
 }
 
-// Factor rows kept in shared memory: as many as the instance's resident CTAs per SM leave
-// room for (the rest stream from L2).  Row i is read at every step after step i, so the
-// first rows carry the most traffic.
-int mix_rows_in_smem(int Qpad, int n, MixVariant v, const DevInfo &di) {
-  const size_t stat = mix_static_smem(v);
-  size_t per_cta = di.smem_per_sm / mix_minb(v);
-  const size_t fixed = stat + 1024 + mix_smem_bytes(Qpad, n, 0, v.RA, v.SR);  // 1 KB reserved per CTA
-  if (per_cta > di.smem_optin) per_cta = di.smem_optin;
-  if (per_cta <= fixed) return 0;
-  const size_t row = (size_t)Qpad * sizeof(float4);
-  const size_t r = (per_cta - fixed) / row;
-  return (int)(r < (size_t)n ? r : (size_t)n);
+// Records and dynamic shared memory of a launch whose largest location has Qpad pairs and n
+// points: a CTA takes its whole share of the SM, the factor rows filling what the state leaves
+// (row i is read at every step after step i, so the first rows carry the most traffic; the
+// rest stream from tensor memory and L2); a state larger than the share takes what it needs.
+void mix_smem(int Qpad, int n, MixVariant v, const DevInfo &di, int *nrec, size_t *smem) {
+  const size_t over = mix_static_smem(v) + 1024;  // 1 KB reserved per CTA
+  size_t share = di.smem_per_sm / mix_minb(v);
+  if (share > di.smem_optin + 1024) share = di.smem_optin + 1024;
+  share -= over;
+  *nrec = v.CL > 1 ? 1 : kRecords;
+  while (*nrec > 1 && mix_state_bytes(Qpad, n, *nrec, v) > share) --*nrec;
+  const size_t need = mix_state_bytes(Qpad, n, *nrec, v);
+  *smem = need > share ? need : share;
+  const size_t all = need + (size_t)n * Qpad * sizeof(int4);  // every row
+  if (*smem > all) *smem = all;
 }
 
 // CTAs of a uniform launch: the instance's resident CTAs per SM (one location each), or in
@@ -580,27 +651,36 @@ int mix_grid(int64_t T, int num_sms, MixVariant v) {
   return (int)(T < g ? (T > 0 ? T : 1) : g);
 }
 
-int mix_cluster_grid(int64_t T, MixVariant v, size_t smem, int num_sms, int *G) {
-  cudaError_t e = cudaFuncSetAttribute(mix_kernel(v), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
+cudaLaunchConfig_t mix_config(MixVariant v, int G, size_t smem, cudaStream_t stream,
+                              cudaLaunchAttribute *attr) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = v.CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(v.CL, 1, 1);
-  cfg.blockDim = dim3(MB, 1, 1);
+  cfg.gridDim = dim3(G, 1, 1);
+  cfg.blockDim = dim3(v.MBT, 1, 1);
   cfg.dynamicSmemBytes = smem;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.stream = stream;
+  if (v.CL > 1) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = v.CL;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  return cfg;
+}
+
+int mix_cluster_grid(int64_t T, MixVariant v, size_t smem, const DevInfo &di, int *G) {
+  const int st = allow_smem(mix_kernel(v), di);
+  if (st) return st;
+  const int num_sms = di.num_sms;
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = mix_config(v, v.CL, smem, nullptr, attr);
   int nc = 0;
-  e = cudaOccupancyMaxActiveClusters(&nc, mix_kernel(v), &cfg);
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&nc, mix_kernel(v), &cfg);
   if (e != cudaSuccess) return cuda_status(e);
   if (nc < 1) return LAGP_ERR_INVALID_ARG;
   int64_t c = nc;
-  c = c < (int64_t)num_sms * LAGP_MIX_MINB / v.CL ? c : (int64_t)num_sms * LAGP_MIX_MINB / v.CL;
+  c = c < (int64_t)num_sms * mix_minb(v) / v.CL ? c : (int64_t)num_sms * mix_minb(v) / v.CL;
   c = c < (T > 0 ? T : 1) ? c : (T > 0 ? T : 1);
   *G = (int)(c * v.CL);
   return LAGP_OK;
@@ -613,8 +693,8 @@ struct MixLayout {
 // [queue | re-score counter | U | Xr | A | design indices | kernel (c) workspace]
 MixLayout mix_layout(int G, int p, int n, int Qpad, int64_t T, int64_t idx_total, int num_sms) {
   MixLayout L;
-  L.u = align_up((size_t)G * n * Qpad * sizeof(float4), 256);
-  L.xr = align_up((size_t)G * p * Qpad * sizeof(float4), 256);
+  L.u = align_up((size_t)G * n * Qpad * sizeof(int4), 256);
+  L.xr = align_up((size_t)G * p * Qpad * sizeof(int4), 256);
   L.a = align_up((size_t)G * n * (n + 2) * sizeof(double), 256);
   L.idx = align_up((size_t)idx_total * sizeof(int32_t), 256);
   L.pred = predict_fp64_workspace_bytes(T, n, num_sms);
@@ -627,7 +707,7 @@ MixLayout mix_layout(int G, int p, int n, int Qpad, int64_t T, int64_t idx_total
 size_t mix_uniform_bytes(int64_t T, int p, int n, int M, int num_sms) {
   size_t best = 0;
   for (int CL = 1; CL <= kMaxCL; CL *= 2) {
-    int64_t G = (int64_t)num_sms * (CL == 1 ? kRingMinB : LAGP_MIX_MINB);
+    int64_t G = (int64_t)num_sms * mix_minb(mix_variant(M, CL, false));
     const int64_t cap = (int64_t)CL * (T > 0 ? T : 1);
     G = G < cap ? G : cap;
     const size_t b = mix_layout((int)G, p, n, mix_qpad(M, CL), T, T * n, num_sms).total;
@@ -636,19 +716,15 @@ size_t mix_uniform_bytes(int64_t T, int p, int n, int M, int num_sms) {
   return best;
 }
 
-// The screen and, per location, the predictive equations on the design it selected: in
-// the same kernel when the matrix fits in its shared memory (paper-2d: 14.43 -> 14.29 ms),
-// else by kernel (c) afterwards (the 8-d workload's n = 100: 139.5 ms either way in its
-// own kernel, 145.5 ms inside the screen from global memory).  The cluster form always
-// leaves them to kernel (c).
+// The screen, then kernel (c) on the designs it selected.
 int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, int32_t *user_idx,
             const DevInfo &di, cudaStream_t stream) {
   P.queue = reinterpret_cast<int *>(w);
   P.rescores = reinterpret_cast<int *>(w + 256);
   char *o = w + 512;
-  P.U = reinterpret_cast<float4 *>(o);
+  P.U = o;
   o += L.u;
-  P.Xr = reinterpret_cast<float4 *>(o);
+  P.Xr = o;
   o += L.xr;
   P.A = reinterpret_cast<double *>(o);
   o += L.a;
@@ -656,88 +732,50 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, int32
   P.idx = user_idx ? user_idx : reinterpret_cast<int32_t *>(o);
   o += L.idx;
   P.CL = v.CL;
-  // tensor-memory rows (one CTA per location): 16, 8 or 4 rows per pair for 1, 2, or 3-4
-  // pairs per thread, so that each thread's rows fit its 64 columns in whole loads of four
-  // rows; none where n leaves no rows past shared memory.
-  // LAGP_MIX_TMEM=0 turns it off (for measurements; no result changes).
-  P.RT = 0;
-  if (v.CL == 1 && mix_env("LAGP_MIX_TMEM") != 0) {
-    const int pp = (P.Qpad + MB - 1) / MB;
-    if (pp <= 4) {
-      v.TM = true;
-      P.RT = 4 * (4 / pp);
-    }
-  }
-  P.R = mix_rows_in_smem(P.Qpad, P.nmax, v, di);
-  if (v.TM && P.nmax <= P.R) {
-    v.TM = false;
-    P.RT = 0;
-    P.R = mix_rows_in_smem(P.Qpad, P.nmax, v, di);
-  }
-  P.fuse_pred = v.RA == 0 && v.CL == 1 &&
-                (size_t)P.R * P.Qpad * sizeof(float4) >= (size_t)P.nmax * (P.nmax + 2) * sizeof(double);
-  const size_t smem = mix_smem_bytes(P.Qpad, P.nmax, P.R, v.RA, v.SR);
+  // LAGP_MIX_TMEM=0 turns the rows in tensor memory off (for measurements; no result changes)
+  P.tmem = mix_env("LAGP_MIX_TMEM") != 0;
+  size_t smem;
+  mix_smem(P.Qpad, P.nmax, v, di, &P.nrec, &smem);
+  P.smem = (int)smem;
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  cudaError_t e = cudaFuncSetAttribute(mix_kernel(v), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return cuda_status(e);
-  if (v.TM) {
-    // every resident CTA holds kTmemCols of the SM's 512 tensor-memory columns: if more
-    // CTAs could be resident than that allows, an allocation would wait for a neighbour to
-    // finish, so such a launch keeps its rows in global memory instead
+  const int st = allow_smem(mix_kernel(v), di);
+  if (st) return st;
+  cudaError_t e;
+  if (v.CL == 1) {
+    // every resident CTA holds its share of the SM's 512 tensor-memory columns; 128 registers
+    // per thread keep the residents at kScrThreads, so an allocation never waits
     int k = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, mix_kernel(v), MB, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, mix_kernel(v), v.MBT, smem);
     if (e != cudaSuccess) return cuda_status(e);
-    if (k * kTmemCols > 512) {
-      v.TM = false;
-      P.RT = 0;
-      e = cudaFuncSetAttribute(mix_kernel(v), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return cuda_status(e);
-    }
+    if (k * tmem_cols(v.MBT) > 512) return LAGP_ERR_CUDA;
   }
   e = cudaMemsetAsync(w, 0, 512, stream);  // work counter and re-score counter
   if (e != cudaSuccess) return cuda_status(e);
-  if (v.CL > 1) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = v.CL;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(G, 1, 1);
-    cfg.blockDim = dim3(MB, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    void *args[] = {&P};
-    e = cudaLaunchKernelExC(&cfg, mix_kernel(v), args);
-    if (e != cudaSuccess) return cuda_status(e);
-  } else if (!v.RA) {
-    if (v.TM)
-      select_mixed_kernel<0, false, false, true><<<G, MB, smem, stream>>>(P);
-    else
-      select_mixed_kernel<0, false, false><<<G, MB, smem, stream>>>(P);
-  } else if (v.SR) {
-    if (v.TM)
-      select_mixed_kernel<RING_A, true, false, true><<<G, MB, smem, stream>>>(P);
-    else
-      select_mixed_kernel<RING_A, true, false><<<G, MB, smem, stream>>>(P);
-  } else {
-    if (v.TM)
-      select_mixed_kernel<RING_A, false, false, true><<<G, MB, smem, stream>>>(P);
-    else
-      select_mixed_kernel<RING_A, false, false><<<G, MB, smem, stream>>>(P);
-  }
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = mix_config(v, G, smem, stream, attr);
+  void *args[] = {&P};
+  e = cudaLaunchKernelExC(&cfg, mix_kernel(v), args);
+  if (e != cudaSuccess) return cuda_status(e);
   g_launches.fetch_add(1);
   e = cudaGetLastError();
-  if (e != cudaSuccess || P.fuse_pred) return cuda_status(e);
+  if (e != cudaSuccess) return cuda_status(e);
   PredictArgs pa;
   pa.X = P.X; pa.Z = P.Z; pa.p = P.pmax; pa.XX = P.XX; pa.T = P.T; pa.n = P.n; pa.nmax = P.nmax;
   pa.theta = P.theta; pa.g = P.g; pa.idx = P.idx; pa.B = P.B;
   pa.B.n_loc = P.n_out;  // adaptive designs: kernel (c) on each location's own size
+  pa.recip = v.fixed;    // FP64: the recursion's own rounding, and no design where it fails
   pa.mean = P.mean; pa.s2 = P.s2; pa.var = P.var; pa.status = P.status;
   return predict_fp64_launch(pa, o, L.pred, stream);
+}
+
+// A batch's instance suits its largest candidate count; the grid is the batch's share of
+// select_max_ctas() CTAs per SM, of that instance's residents.
+MixVariant mix_batch_variant(const BatchLaunch &b) { return mix_variant(b.Mmax, 1, b.precision == LAGP_FP64); }
+int mix_batch_grid(const BatchLaunch &b, int num_sms) {
+  const int most = select_max_ctas(b.method, b.precision);
+  const int ctas = b.ctas_per_sm < 1 || b.ctas_per_sm > most ? most : b.ctas_per_sm;
+  const int64_t g = (int64_t)num_sms * mix_minb(mix_batch_variant(b)) * ctas / most;
+  return (int)(g < 1 ? 1 : g < b.T ? g : b.T);
 }
 
 }  // namespace
@@ -755,12 +793,14 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  const MixVariant v = mix_variant(a.n, a.M, mix_cluster_size(a.n, a.M), di);
+  const MixVariant v = mix_variant(a.M, a.precision == LAGP_FP64 ? 1 : mix_cluster_size(), a.precision == LAGP_FP64);
   const int Qpad = mix_qpad(a.M, v.CL);
   int G = mix_grid(a.T, di.num_sms, v);
   if (v.CL > 1) {
-    const int R = mix_rows_in_smem(Qpad, a.n, v, di);
-    st = mix_cluster_grid(a.T, v, mix_smem_bytes(Qpad, a.n, R, v.RA, v.SR), di.num_sms, &G);
+    int nrec;
+    size_t smem;
+    mix_smem(Qpad, a.n, v, di, &nrec, &smem);
+    st = mix_cluster_grid(a.T, v, smem, di, &G);
     if (st) return st;
   }
   const MixLayout L = mix_layout(G, a.p, a.n, Qpad, a.T, a.T * a.n, di.num_sms);
@@ -777,20 +817,21 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
   return mix_run(P, v, L, G, static_cast<char *>(ws), a.idx, di, stream);
 }
 
-size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b, int G) {
+size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b) {
   DevInfo di;
   const int sms = dev_info(&di) == LAGP_OK ? di.num_sms : 152;
-  return mix_layout(G, b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.T, b.idx_total, sms).total;
+  return mix_layout(mix_batch_grid(b, sms), b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.T, b.idx_total, sms).total;
 }
 
-int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, int G,
-                              cudaStream_t stream) {
+// (Locations grouped by candidate count, one launch of a fitting instance each, measured slower:
+// 3000 locations of up to 4000 candidates 90.6 -> 97.1 ms, the launches' tails.)
+int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream) {
   DevInfo di;
   int st = dev_info(&di);
   if (st) return st;
   st = exp_table_upload();  // this translation unit's copy of the exp constants
   if (st) return st;
-  const int Qpad = mix_qpad(b.Mmax, 1);
+  const int G = mix_batch_grid(b, di.num_sms), Qpad = mix_qpad(b.Mmax, 1);
   const MixLayout L = mix_layout(G, b.pmax, b.nmax, Qpad, b.T, b.idx_total, di.num_sms);
   if (ws_bytes < L.total) return LAGP_ERR_INVALID_ARG;
   MixParams P;
@@ -802,9 +843,7 @@ int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, i
   P.start = nullptr; P.nstart = 0;
   P.r_min = 0.0; P.n_out = nullptr;
   P.mean = b.mean; P.s2 = b.s2; P.var = b.var; P.status = b.status;
-  // batches keep one CTA per location (their tuner chooses the CTAs per SM)
-  MixVariant v = mix_variant(b.nmax, b.Mmax, 1, di);
-  return mix_run(P, v, L, G, static_cast<char *>(ws), b.idx, di, stream);
+  return mix_run(P, mix_batch_variant(b), L, G, static_cast<char *>(ws), b.idx, di, stream);
 }
 
 int select_mixed_prepare() {
