@@ -1,7 +1,11 @@
-"""NN by the predictive kernel alone against the FP64 recursion (which the no-allocation entry
-point runs on the same inputs): the predictive kernel makes the recursion's operations in its
-order, so designs, statuses and values must be the same bit for bit.  Sizes at the edges of
-the predictive kernel's group form (n = 208) and its teams (64 threads)."""
+"""The FP64 ALC designs by the fixed-point screen, and NN by the predictive kernel alone,
+against the FP64 recursion (which the no-allocation entry point runs on the same inputs): every
+decision of the screen that is not clear by its margin is taken in the recursion's own
+arithmetic, and the predictive kernel makes the recursion's operations in its order, so
+designs, statuses and values must be the same bit for bit.  Sizes at the edges of the screen's
+instances (64, 128, 256 candidate pairs), of the predictive kernel's group form (n = 208) and
+its teams (64 threads), odd candidate counts, no greedy step at all, and the options that
+change the number format (wide spread, large and tiny nuggets)."""
 from __future__ import annotations
 
 import numpy as np
@@ -12,13 +16,15 @@ from paper_1303_0383_gb300 import lagp
 pytestmark = pytest.mark.gpu
 
 
-def _both(N, p, T, n0, n, M, theta, g, method, seed):
+def _both(N, p, T, n0, n, M, theta, g, method, seed, poison=None, spread=1.0):
     import torch
     rng = np.random.default_rng(seed)
-    X = rng.random((N, p))
+    X = rng.random((N, p)) * spread
     Z = np.sin(3 * X[:, 0]) + X.sum(1)
-    XX = rng.random((T, p))
+    XX = rng.random((T, p)) * spread
     near = np.argsort(((XX[:, None] - X[None]) ** 2).sum(-1), axis=1, kind="stable")[:, :M]
+    if poison is not None:
+        X[near[0, M // 2], 0] = poison
     d = lambda a: torch.as_tensor(np.ascontiguousarray(a)).cuda()
     X, Z, XX, cand = d(X), d(Z), d(XX), d(near.astype(np.int32))
     res = []
@@ -38,6 +44,27 @@ def _both(N, p, T, n0, n, M, theta, g, method, seed):
     for k in res[0]:
         assert np.array_equal(res[0][k], res[1][k], equal_nan=k not in ("idx", "status")), k
     return res[0]
+
+
+@pytest.mark.parametrize("N,p,T,n0,n,M", [
+    (40, 1, 3, 3, 12, 16), (600, 2, 5, 6, 6, 255), (300, 2, 4, 6, 40, 256), (300, 2, 4, 6, 41, 257),
+    (700, 3, 9, 5, 30, 511), (700, 3, 9, 5, 30, 512), (700, 8, 3, 7, 33, 513), (1200, 2, 2, 3, 20, 1025),
+    (64, 2, 3, 4, 64, 64), (400, 2, 3, 6, 209, 301), (4200, 2, 1, 6, 12, 4097)])
+def test_fp64_alc_sizes(N, p, T, n0, n, M):
+    r = _both(N, p, T, n0, n, M, 0.3, 1e-5, "alc", 11 * M + n)
+    assert (r["status"] == 0).all()
+
+
+@pytest.mark.parametrize("theta,g,spread", [
+    (0.5, 0.9, 1.0), (0.5, 3.0, 1.0), (0.5, 2.0 ** -30, 1.0), (0.5, 2.0 ** -31, 1.0), (1e-3, 1e-6, 1.0),
+    (0.5, 1e-5, 40.0), (0.5, 1e-5, 3e3), (1e3, 1e-6, 1.0), (0.2, 1e-5, 1e-4)])
+def test_fp64_alc_formats(theta, g, spread):
+    _both(500, 2, 6, 5, 30, 300, theta, g, "alc", 5, spread=spread)
+
+
+@pytest.mark.parametrize("poison", [np.inf, np.nan, 1e200])
+def test_fp64_alc_values_out_of_range(poison):
+    _both(500, 2, 4, 5, 20, 200, 0.3, 1e-5, "alc", 6, poison=poison)
 
 
 @pytest.mark.parametrize("T,n,M", [(1, 3, 3), (700, 50, 60), (7, 64, 64), (310, 65, 70), (5, 208, 210),
