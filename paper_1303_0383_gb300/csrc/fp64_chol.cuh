@@ -30,9 +30,11 @@ __device__ __forceinline__ int tri_row(int e) {
 // recip: the matrix entries (not the extra columns) are multiplied by 1 / l_kk instead of
 // divided by l_kk: the rounding of the FP64 recursion's candidate rows (select.cu), so a
 // design's rows come out bit for bit as that recursion forms them.
+// turn: the warp that takes the pivots.  Warp w of every CTA runs on sub-partition w mod 4, so
+// CTAs that share an SM should have them taken by different ones.
 __device__ void chol_flat_fp64(double *A, int n, int lda, int naug, double *rl, int *fail,
-                               bool recip = false) {
-  const int tid = threadIdx.x, nt = blockDim.x;
+                               bool recip = false, int turn = 0) {
+  const int nt = blockDim.x, first = (int)threadIdx.x - 32 * turn, tid = first < 0 ? first + nt : first;
   __syncthreads();
   if (tid == 0) {
     const double d0 = A[0];

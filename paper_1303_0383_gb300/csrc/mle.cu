@@ -57,14 +57,22 @@ struct MleParams {
   int *queue;
 };
 
-// Per-CTA buffers: three n x n FP64 matrices (L then K^-1, Kd, L^-1), four FP64 vectors
-// and the design's coordinates (up to kMaxP per point).  Squared distances are recomputed
-// from the coordinates where needed (p operations each, in the same order every time),
-// which leaves room for three CTAs per SM at n = 50: the Cholesky's pivot chain is
-// sequential, and more locations in flight hide it.
+// Per-CTA buffers: two squares of rows of lda doubles (odd: a column's entries lie in different
+// banks), each a symmetric or triangular matrix in its lower triangle, diagonal included,
+// and another in its upper one, a packed triangle, and four vectors.
+//   S1  lower K, its Cholesky factor L, then K^-1;  upper the squared distances
+//   S2  lower Kd;  upper X = L^-1, transposed (x_ii = 1 / l_ii is in rl), then A_ab
+//   S3  the design's coordinates, then Kdd, then A_ba
+// so that four CTAs share an SM at n = 50 (three with full matrices: 500 locations were a wave
+// and a tenth): the factorisation's pivot chain is sequential, and more locations in flight
+// hide it.  Squared distances are formed once per location, Kdd once per iteration.  GB300, two
+// stages over 500 8-d locations, n = 50, the MLE of the first among them: 11.99 -> 8.22 ms.
+__host__ __device__ constexpr int mle_lda(int n) { return n | 1; }
+__host__ __device__ constexpr size_t mle_s3_words(int n) {
+  return (size_t)n * (n + 1) / 2 > (size_t)n * kMaxP ? (size_t)n * (n + 1) / 2 : (size_t)n * kMaxP;
+}
 size_t mle_set_bytes(int n) {
-  const size_t nn = (size_t)n * n;
-  return nn * 3 * sizeof(double) + (size_t)n * (4 + kMaxP) * sizeof(double);
+  return (2 * (size_t)n * mle_lda(n) + mle_s3_words(n) + 4 * (size_t)n) * sizeof(double);
 }
 
 // Lane 0's shuffle-tree sum of v over its warp.
@@ -73,23 +81,25 @@ __device__ __forceinline__ double warp_tree_sum(double v) {
   return v;
 }
 
-__global__ void __launch_bounds__(LB) mle_fp64_kernel(MleParams P) {
+__global__ void __launch_bounds__(LB, 4) mle_fp64_kernel(MleParams P) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nmax = P.n;
   unsigned char *base = P.in_smem ? smraw : P.slots + (size_t)blockIdx.x * P.slot_bytes;
-  const size_t nn = (size_t)nmax * nmax;
-  double *Lm = reinterpret_cast<double *>(base);  // K, its Cholesky factor L, then K^-1
-  double *Kd = Lm + nn;
-  double *Ki = Kd + nn;
-  double *Y = Ki + nn, *w = Y + nmax, *kdw = w + nmax, *rl = kdw + nmax;
-  double *xd = rl + nmax;    // nmax x p coordinates of the design
+  const int lda = mle_lda(nmax);
+  double *S1 = reinterpret_cast<double *>(base);
+  double *S2 = S1 + (size_t)nmax * lda, *S3 = S2 + (size_t)nmax * lda;
+  double *Y = S3 + mle_s3_words(nmax), *w = Y + nmax, *kdw = w + nmax, *rl = kdw + nmax;
   __shared__ double etab[64];
   __shared__ double red[kSums][LB / 32];
   __shared__ double sh_th, sh_lo, sh_hi;
   __shared__ int sh_loc, sh_fail, sh_done, sh_lo_open, sh_hi_open, sh_it, sh_st;
   const int tid = threadIdx.x;
   if (tid < 64) etab[tid] = c_exp.tab[tid];
-  const int n = P.n, p = P.p, lda = n;
+  const int n = P.n, p = P.p, ntri = n * (n + 1) / 2;
+  // one pivot warp per sub-partition for the CTAs of an SM (dealt to the SMs in turn)
+  unsigned nsm;
+  asm("mov.u32 %0, %%nsmid;" : "=r"(nsm));
+  const int turn = (int)(blockIdx.x / nsm) & 3;
 
   for (;;) {
     __syncthreads();
@@ -112,85 +122,82 @@ __global__ void __launch_bounds__(LB) mle_fp64_kernel(MleParams P) {
     __syncthreads();
     if (!sh_fail) {
       for (int i = tid; i < n; i += LB) Y[i] = P.Z[d[i]];
-      for (int e = tid; e < n * p; e += LB) xd[e] = P.X[(int64_t)d[e / p] * p + e % p];
+      for (int e = tid; e < n * p; e += LB) S3[e] = P.X[(int64_t)d[e / p] * p + e % p];
     }
     __syncthreads();  // the coordinates are read by other threads below
-    // squared distance of design points a and b
-    auto r2of = [&](int a, int b) {
-      double r2 = 0.0;
-      for (int k = 0; k < p; k++) {
-        const double t = xd[a * p + k] - xd[b * p + k];
-        r2 = fma(t, t, r2);
+    if (!sh_fail)
+      for (int e = tid; e < ntri; e += LB) {
+        const int a = tri_row(e), b = e - a * (a + 1) / 2;
+        if (a == b) continue;
+        double r2 = 0.0;
+        for (int k = 0; k < p; k++) {
+          const double t = S3[a * p + k] - S3[b * p + k];
+          r2 = fma(t, t, r2);
+        }
+        S1[b * lda + a] = r2;
       }
-      return r2;
-    };
+    __syncthreads();
     while (!sh_fail && !sh_done) {
       const double th = sh_th;
       const double tinv = 1.0 / th, tinv2 = tinv * tinv;
-      // K (lower triangle) and Kd (full): one exp per pair a > b, mirrored
-      const int ntri = n * (n + 1) / 2;
+      // K, Kd and Kdd: one exp per pair a > b
       for (int e = tid; e < ntri; e += LB) {
         const int a = tri_row(e), b = e - a * (a + 1) / 2;
+        double r2 = 0.0, kd = 0.0;
         if (a == b) {
-          Lm[a * lda + a] = 1.0 + P.g;
-          Kd[a * lda + a] = 0.0;
+          S1[a * lda + a] = 1.0 + P.g;
         } else {
-          const double r2 = r2of(a, b);
+          r2 = S1[b * lda + a];
           const double k = exp_nonpos(-r2 * tinv, etab);
-          Lm[a * lda + b] = k;
-          const double kd = k * r2 * tinv2;
-          Kd[a * lda + b] = kd;
-          Kd[b * lda + a] = kd;
+          S1[a * lda + b] = k;
+          kd = k * r2 * tinv2;
         }
+        S2[a * lda + b] = kd;
+        S3[e] = kd * fma(r2, tinv2, -2.0 * tinv);
       }
-      chol_flat_fp64(Lm, n, lda, 0, rl, &sh_fail);
+      chol_flat_fp64(S1, n, lda, 0, rl, &sh_fail, false, turn);
       if (sh_fail) break;
-      // X = L^-1 (lower triangle, in Ki's storage): x_ic = -(sum_{c<=m<i} l_im x_mc) / l_ii,
-      // x_ii = 1 / l_ii.  Right-looking: at step m every entry (i > m, c <= m) takes its
-      // term l_im x_mc -- the same terms in the same order as the row-by-row sums -- and
-      // the thread that adds the last term of row m + 1 finishes that entry, so a step is
-      // one barrier and all threads share its FP64 work.  Row m + 1 runs in a loop of its
-      // own: in the shared loop its multiply by 1 / l_ii would be a predicated FP64
-      // instruction issued by every warp.
-      double *Xb = Ki;
-      for (int e = tid; e < ntri; e += LB) {
-        const int a = tri_row(e), b = e - a * (a + 1) / 2;
-        Xb[a * lda + b] = (a == b) ? rl[a] : 0.0;
-      }
-      __syncthreads();
+      // X = L^-1: x_ic = -(sum_{c<=m<i} l_im x_mc) / l_ii, x_ii = 1 / l_ii.  Right-looking: at
+      // step m every entry (i > m, c <= m) takes its term l_im x_mc -- the same terms in the
+      // same order as the row-by-row sums -- and the thread that adds the last term of row
+      // m + 1 finishes that entry, so a step is one barrier and all threads share its FP64
+      // work.  Row m + 1 runs in a loop of its own: in the shared loop its multiply by 1 / l_ii
+      // would be a predicated FP64 instruction issued by every warp.
       for (int m = 0; m < n - 1; m++) {
         const int w1 = m + 1, cnt = (n - 1 - m) * w1;
         {  // row m + 1: its last term, then the division by its pivot
           const int i = m + 1;
-          for (int c = tid; c < w1; c += LB)
-            Xb[i * lda + c] = -fma(Lm[i * lda + m], Xb[m * lda + c], Xb[i * lda + c]) * rl[i];
+          for (int c = tid; c < w1; c += LB) {
+            const double x = c == m ? rl[m] : S2[c * lda + m], s = c == m ? 0.0 : S2[c * lda + i];
+            S2[c * lda + i] = -fma(S1[i * lda + m], x, s) * rl[i];
+          }
         }
         for (int e = w1 + tid; e < cnt; e += LB) {
           const int i = m + 1 + e / w1, c = e % w1;
-          Xb[i * lda + c] = fma(Lm[i * lda + m], Xb[m * lda + c], Xb[i * lda + c]);
+          const double x = c == m ? rl[m] : S2[c * lda + m], s = c == m ? 0.0 : S2[c * lda + i];
+          S2[c * lda + i] = fma(S1[i * lda + m], x, s);
         }
         __syncthreads();
       }
-      // K^-1 = X^T X (both triangles) into L's storage, which is no longer needed
-      double *KiM = Lm;
+      // K^-1 = X^T X into L's storage, which is no longer needed
       for (int e = tid; e < ntri; e += LB) {
         const int a = tri_row(e), b = e - a * (a + 1) / 2;
-        double s = 0.0;
-        for (int m = a; m < n; m++) s = fma(Xb[m * lda + a], Xb[m * lda + b], s);
-        KiM[a * lda + b] = s;
-        KiM[b * lda + a] = s;
+        double s = fma(rl[a], a == b ? rl[a] : S2[b * lda + a], 0.0);
+        for (int m = a + 1; m < n; m++) s = fma(S2[a * lda + m], S2[b * lda + m], s);
+        S1[a * lda + b] = s;
       }
       __syncthreads();
-      // w = K^-1 Y, then Kd w
+      // w = K^-1 Y, then Kd w (entry (a, b) of a symmetric matrix: along row a up to the
+      // diagonal, then down column a)
       for (int a = tid; a < n; a += LB) {
         double s = 0.0;
-        for (int b = 0; b < n; b++) s = fma(KiM[a * lda + b], Y[b], s);
+        for (int b = 0, q = a * lda; b < n; q += b < a ? 1 : lda, b++) s = fma(S1[q], Y[b], s);
         w[a] = s;
       }
       __syncthreads();
       for (int a = tid; a < n; a += LB) {
         double s = 0.0;
-        for (int b = 0; b < n; b++) s = fma(Kd[a * lda + b], w[b], s);
+        for (int b = 0, q = a * lda; b < n; q += b < a ? 1 : lda, b++) s = fma(S2[q], w[b], s);
         kdw[a] = s;
       }
       __syncthreads();
@@ -200,9 +207,8 @@ __global__ void __launch_bounds__(LB) mle_fp64_kernel(MleParams P) {
         psi = fma(Y[a], w[a], psi);
         q3 = fma(w[a], kdw[a], q3);
         double sdd = 0.0, sq2 = 0.0, st1 = 0.0, st3 = 0.0;
-        for (int b = 0; b < n; b++) {
-          const double kd = Kd[a * lda + b], kdd = kd * (r2of(a, b) * tinv2 - 2.0 * tinv);
-          const double ki = KiM[a * lda + b];
+        for (int b = 0, q = a * lda, t = a * (a + 1) / 2; b < n; q += b < a ? 1 : lda, b++, t += b > a ? b : 1) {
+          const double kd = S2[q], kdd = S3[t], ki = S1[q];
           sdd = fma(kdd, w[b], sdd);
           sq2 = fma(ki, kdw[b], sq2);
           st1 = fma(ki, kd, st1);
@@ -219,27 +225,27 @@ __global__ void __launch_bounds__(LB) mle_fp64_kernel(MleParams P) {
       // enters l'' only, which sets the Newton step, not the root l' = 0 the iteration
       // converges to.  K^-1 and Kd are converted in place (their FP64 uses are done), one
       // float-float pair per FP64 slot.
-      float2 *Kif = reinterpret_cast<float2 *>(KiM), *Kdf = reinterpret_cast<float2 *>(Kd);
-      for (int e = tid; e < n * n; e += LB) {
-        const ff ki = ff_from_double(KiM[e]), kd = ff_from_double(Kd[e]);
-        Kif[e] = make_float2(ki.h, ki.l);
-        Kdf[e] = make_float2(kd.h, kd.l);
+      float2 *Kif = reinterpret_cast<float2 *>(S1), *Kdf = reinterpret_cast<float2 *>(S2);
+      for (int e = tid; e < ntri; e += LB) {
+        const int a = tri_row(e), q = a * lda + e - a * (a + 1) / 2;
+        const ff ki = ff_from_double(S1[q]), kd = ff_from_double(S2[q]);
+        Kif[q] = make_float2(ki.h, ki.l);
+        Kdf[q] = make_float2(kd.h, kd.l);
       }
       __syncthreads();
-      // The pairs a <= b, all lanes busy: (a == b ? 1 : 2) A_ab into slot (a, b) and A_ba into
-      // slot (b, a) of the dead L^-1 storage (for a == b both are A_aa, in one slot).
+      // The pairs a <= b, all lanes busy: (a == b ? 1 : 2) A_ab and A_ba (for a == b both are
+      // A_aa)
       for (int e = tid; e < ntri; e += LB) {
         const int b = tri_row(e), a = e - b * (b + 1) / 2;
         ffacc sab{0.0f, 0.0f}, sba{0.0f, 0.0f};
-        for (int m = 0; m < n; m++) {
-          const float2 x1 = Kif[a * lda + m], y1 = Kdf[m * lda + b];
-          const float2 x2 = Kif[b * lda + m], y2 = Kdf[m * lda + a];
+        for (int m = 0, qa = a * lda, qb = b * lda; m < n; qa += m < a ? 1 : lda, qb += m < b ? 1 : lda, m++) {
+          const float2 x1 = Kif[qa], y1 = Kdf[qb], x2 = Kif[qb], y2 = Kdf[qa];
           ffacc_add_prod(sab, ff{x1.x, x1.y}, ff{y1.x, y1.y});
           ffacc_add_prod(sba, ff{x2.x, x2.y}, ff{y2.x, y2.y});
         }
         const double vab = (double)sab.h + (double)sab.l, vba = (double)sba.h + (double)sba.l;
-        Xb[a * lda + b] = (a == b ? 1.0 : 2.0) * vab;
-        if (a != b) Xb[b * lda + a] = vba;
+        if (a != b) S2[a * lda + b] = 2.0 * vab;
+        S3[e] = vba;
       }
       __syncthreads();
       // each thread adds its pairs in the order of the row-major (a, b) scan
@@ -247,7 +253,8 @@ __global__ void __launch_bounds__(LB) mle_fp64_kernel(MleParams P) {
       for (int e = tid; e < n * n; e += LB) {
         const int a = e / n, b = e % n;
         if (b < a) continue;
-        t2p = fma(Xb[a * lda + b], Xb[b * lda + a], t2p);
+        const double v = S3[b * (b + 1) / 2 + a];
+        t2p = fma(a == b ? v : S2[a * lda + b], v, t2p);
       }
       // The seven block sums: a shuffle tree per warp, then thread 0 adds the warp totals in
       // warp order.  The six row sums are exactly +0.0 in a warp none of whose threads holds
