@@ -132,6 +132,7 @@ int select_mspe_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStrea
 size_t select_mspe_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms);
 int select_mspe_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream);
 #define LAGP_MSPE_MIX_CTAS_PER_SM 2  // resident CTAs per SM of the mixed MSPE kernel
+#define LAGP_MSPE_CTAS_PER_SM 2      // resident CTAs per SM of the FP64 MSPE kernel
 
 // Batched launch of kernels (b)+(c): per-location tables in device memory (batch.cuh),
 // one persistent launch of G = ctas_per_sm x SMs CTAs over the cost-ordered queue.

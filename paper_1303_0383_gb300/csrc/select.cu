@@ -383,7 +383,7 @@ int select_launch_on_grid(const SelectArgs &a, void *ws, size_t ws_bytes, int G,
 }
 
 int select_max_ctas(int32_t method, int32_t precision) {
-  if (method == LAGP_MSPE) return precision == LAGP_MIXED ? LAGP_MSPE_MIX_CTAS_PER_SM : 1;
+  if (method == LAGP_MSPE) return precision == LAGP_MIXED ? LAGP_MSPE_MIX_CTAS_PER_SM : LAGP_MSPE_CTAS_PER_SM;
   return 2;
 }
 

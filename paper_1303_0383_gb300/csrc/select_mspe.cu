@@ -27,6 +27,11 @@
 namespace lagp {
 namespace {
 
+// Bound by the FP64 pipe where a candidate's rows are updated, and by the chains of the O(j^2)
+// design step elsewhere, which leave it idle: two CTAs per SM fill each other's gaps (their
+// rows exceed L2, 243 MB at n = 50, M = 1000, but DRAM has room: 3 ms of 19), and Kd's and Kdd's
+// products run in threads of their own.  GB300, 1000 8-d locations, n = 50 of 1000, whole call:
+// 21.12 -> 18.91 ms; 400 at n = 100 of 2000: 48.0 -> 41.0 ms.
 constexpr int TB = 256;  // threads per CTA
 
 struct MspeParams {
@@ -45,7 +50,7 @@ struct MspeParams {
   double *U, *Ud;     // slots of n x Mpad
   double *Xc;         // slots of p x Mpad
   double *cs;         // slots of 4 x Mpad: kdz, pd, q, m per candidate
-  double *Li, *Kd, *Kdd, *Q;  // slots of n x n
+  double *Li, *Kd, *Kdd;  // slots of n x n
   int *queue;
   const int32_t *start;  // saved start designs (T x nstart design indices), or nullptr
   int nstart;
@@ -55,7 +60,7 @@ __device__ __forceinline__ bool j_better(double a, int ra, double b, int rb) {
   return a < b || (a == b && ra < rb);
 }
 
-__global__ void __launch_bounds__(TB, 1) select_mspe_kernel(MspeParams P) {
+__global__ void __launch_bounds__(TB, LAGP_MSPE_CTAS_PER_SM) select_mspe_kernel(MspeParams P) {
   extern __shared__ __align__(16) double sm[];
   const int Mpad = P.Mpad, nn = P.nmax;  // nn: row stride of the n x n slot matrices
   double *v = sm;               // Mpad: v_j(c)
@@ -70,7 +75,8 @@ __global__ void __launch_bounds__(TB, 1) select_mspe_kernel(MspeParams P) {
   double *r = yt + nn;          // nn: Q ytil
   double *t1 = r + nn;          // nn: Kd Li[j]^T
   double *t2 = t1 + nn;         // nn: Kdd Li[j]^T
-  int *dr = reinterpret_cast<int *>(t2 + nn);  // nn: ranks of the design
+  double *lrow = t2 + nn;       // nn: row j of L^{-1}
+  int *dr = reinterpret_cast<int *>(lrow + nn);  // nn: ranks of the design
   unsigned char *used = reinterpret_cast<unsigned char *>(dr + nn);  // Mpad
   __shared__ double etab[64];
   __shared__ double xs[kMaxP], xl[kMaxP];
@@ -90,7 +96,6 @@ __global__ void __launch_bounds__(TB, 1) select_mspe_kernel(MspeParams P) {
   double *Li = P.Li + (size_t)blockIdx.x * nn * nn;
   double *Kd = P.Kd + (size_t)blockIdx.x * nn * nn;
   double *Kdd = P.Kdd + (size_t)blockIdx.x * nn * nn;
-  double *Q = P.Q + (size_t)blockIdx.x * nn * nn;
 
   for (;;) {
     __syncthreads();
@@ -195,6 +200,7 @@ __global__ void __launch_bounds__(TB, 1) select_mspe_kernel(MspeParams P) {
           li = -acc * inv;
         }
         Li[(size_t)j * nn + i] = li;
+        lrow[i] = li;
         double kd = 0.0, kdd = 0.0;
         if (i < j) {
           const double *xi = L.X + (int64_t)cnd[dr[i]] * p;
@@ -212,29 +218,28 @@ __global__ void __launch_bounds__(TB, 1) select_mspe_kernel(MspeParams P) {
       }
       __syncthreads();
       // t1 = Kd Li[j]^T, t2 = Kdd Li[j]^T over rows a <= j (symmetric: entry (a,c) at row max)
-      for (int a = tid; a <= j; a += TB) {
-        double s1 = 0.0, s2 = 0.0;
+      for (int e = tid; e < 2 * (j + 1); e += TB) {
+        const bool dd = e > j;
+        const int a = dd ? e - j - 1 : e;
+        const double *K = (dd ? Kdd : Kd) + (size_t)a * nn;  // along row a, then down column a
+        double s1 = 0.0;
+#pragma unroll 4
         for (int c = 0; c <= j; c++) {
-          const int hi = a > c ? a : c, lo = a > c ? c : a;
-          const double lj = Li[(size_t)j * nn + c];
-          s1 = fma(Kd[(size_t)hi * nn + lo], lj, s1);
-          s2 = fma(Kdd[(size_t)hi * nn + lo], lj, s2);
+          s1 = fma(*K, lrow[c], s1);
+          K += c < a ? 1 : nn;
         }
-        t1[a] = s1;
-        t2[a] = s2;
+        (dd ? t2 : t1)[a] = s1;
       }
       __syncthreads();
       // row j of Q and R: (Li t)[b] = sum_{a <= b} Li[b][a] t[a]
-      for (int b = tid; b <= j; b += TB) {
-        double s1 = 0.0, s2 = 0.0;
-        for (int a = 0; a <= b; a++) {
-          const double l = Li[(size_t)b * nn + a];
-          s1 = fma(l, t1[a], s1);
-          s2 = fma(l, t2[a], s2);
-        }
-        Q[(size_t)j * nn + b] = s1;
-        qrow[b] = s1;
-        rrow[b] = s2;
+      for (int e = tid; e < 2 * (j + 1); e += TB) {
+        const bool dd = e > j;
+        const int b = dd ? e - j - 1 : e;
+        const double *l = Li + (size_t)b * nn, *t = dd ? t2 : t1;
+        double s1 = 0.0;
+#pragma unroll 4
+        for (int a = 0; a <= b; a++) s1 = fma(l[a], t[a], s1);
+        (dd ? rrow : qrow)[b] = s1;
       }
       __syncthreads();
       // r = Q ytil: old entries gain Q[j][i] ytil_j; entry j is row j of Q dotted with ytil
@@ -388,7 +393,7 @@ __global__ void __launch_bounds__(TB, 1) select_mspe_kernel(MspeParams P) {
 }
 
 int mspe_grid(int64_t T, int num_sms) {
-  const int64_t g = num_sms;
+  const int64_t g = (int64_t)num_sms * LAGP_MSPE_CTAS_PER_SM;
   return (int)(T < g ? (T > 0 ? T : 1) : g);
 }
 
@@ -396,7 +401,7 @@ struct MspeLayout {
   size_t u, ud, xc, cs, nn, idx, pred, total;
 };
 
-// [queue | U | Ud | Xc | cs | Li, Kd, Kdd, Q | design indices | kernel (c) workspace]
+// [queue | U | Ud | Xc | cs | Li, Kd, Kdd | design indices | kernel (c) workspace]
 MspeLayout mspe_layout(int G, int p, int n, int M, int64_t T, int64_t idx_total, int num_sms) {
   const size_t Mpad = align_up((size_t)M, 32);
   MspeLayout L;
@@ -407,12 +412,12 @@ MspeLayout mspe_layout(int G, int p, int n, int M, int64_t T, int64_t idx_total,
   L.nn = align_up((size_t)G * n * n * sizeof(double), 256);
   L.idx = align_up((size_t)idx_total * sizeof(int32_t), 256);
   L.pred = predict_fp64_workspace_bytes(T, n, num_sms);
-  L.total = 256 + L.u + L.ud + L.xc + L.cs + 4 * L.nn + L.idx + L.pred;
+  L.total = 256 + L.u + L.ud + L.xc + L.cs + 3 * L.nn + L.idx + L.pred;
   return L;
 }
 
 size_t mspe_smem_bytes(int Mpad, int n) {
-  return (size_t)(2 * Mpad + 10 * n) * sizeof(double) + (size_t)n * sizeof(int) +
+  return (size_t)(2 * Mpad + 11 * n) * sizeof(double) + (size_t)n * sizeof(int) +
          align_up((size_t)Mpad, 16);
 }
 
@@ -431,7 +436,6 @@ int mspe_run(MspeParams P, const MspeLayout &L, int G, char *w, int32_t *user_id
   P.Li = reinterpret_cast<double *>(w + off); off += L.nn;
   P.Kd = reinterpret_cast<double *>(w + off); off += L.nn;
   P.Kdd = reinterpret_cast<double *>(w + off); off += L.nn;
-  P.Q = reinterpret_cast<double *>(w + off); off += L.nn;
   P.idx = user_idx ? user_idx : reinterpret_cast<int32_t *>(w + off);
   off += L.idx;
   const size_t smem = mspe_smem_bytes(P.Mpad, P.nmax);
@@ -465,8 +469,12 @@ int select_mspe_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStrea
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  const int G = mspe_grid(a.T, di.num_sms);
-  const MspeLayout L = mspe_layout(G, a.p, a.n, a.M, a.T, a.T * a.n, di.num_sms);
+  int G = mspe_grid(a.T, di.num_sms);
+  MspeLayout L = mspe_layout(G, a.p, a.n, a.M, a.T, a.T * a.n, di.num_sms);
+  if (ws_bytes < L.total && G > di.num_sms) {  // one CTA per SM in a smaller workspace
+    G = di.num_sms;
+    L = mspe_layout(G, a.p, a.n, a.M, a.T, a.T * a.n, di.num_sms);
+  }
   if (ws_bytes < L.total) return LAGP_ERR_INVALID_ARG;
   MspeParams P;
   P.X = a.X; P.Z = a.Z; P.p = a.p; P.XX = a.XX; P.T = a.T; P.cand = a.cand;

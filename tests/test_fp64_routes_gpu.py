@@ -5,7 +5,8 @@ arithmetic, and the predictive kernel makes the recursion's operations in its or
 designs, statuses and values must be the same bit for bit.  Sizes at the edges of the screen's
 instances (64, 128, 256 candidate pairs), of the predictive kernel's group form (n = 208) and
 its teams (64 threads), odd candidate counts, no greedy step at all, and the options that
-change the number format (wide spread, large and tiny nuggets)."""
+change the number format (wide spread, large and tiny nuggets).  And FP64 MSPE in a workspace
+of fewer CTAs, whose results are the same."""
 from __future__ import annotations
 
 import numpy as np
@@ -77,3 +78,21 @@ def test_nn_sizes(T, n, M):
 def test_nn_failed_factorisation():
     r = _both(300, 2, 9, 3, 60, 60, 1e4, 0.0, "nn", 3)  # correlations of 1: no factor
     assert (r["status"] != 0).any()
+
+
+def test_mspe_in_a_smaller_workspace():
+    import torch
+    T, n, M = 400, 20, 200
+    rng = np.random.default_rng(8)
+    X, XX = torch.as_tensor(rng.random((900, 2))).cuda(), torch.as_tensor(rng.random((T, 2))).cuda()
+    Z = torch.sin(3 * X[:, 0]) + X.sum(1)
+    cand = torch.argsort(((XX[:, None] - X[None]) ** 2).sum(-1), dim=1, stable=True)[:, :M].to(torch.int32).contiguous()
+    full = lagp.lagp_select_workspace_bytes(T, 2, n, M, "mspe")
+    res = []
+    for nbytes in (full, full * 6 // 10):
+        mean, s2 = (torch.full((T,), 7.0, dtype=torch.float64, device="cuda") for _ in range(2))
+        idx = torch.full((T, n), -7, dtype=torch.int32, device="cuda")
+        lagp.lagp_select_dev(X, Z, XX, cand, 6, n, 0.3, 1e-4, "mspe", "fp64", mean, s2, None, idx, None,
+                             lagp.workspace(nbytes))
+        res.append((mean, s2, idx))
+    assert all(torch.equal(a, b) for a, b in zip(*res)) and bool(torch.isfinite(res[0][0]).all())
