@@ -34,6 +34,9 @@ sys.path.insert(0, ROOT)
 METRIC = "local-GP predictions/sec (n=50, 1000 cand) FP64 plain vs mixed; serving p99 ms"
 UNIT = "predictions/s"
 FP64_PEAK_TFLOPS_DERIVED = 152 * 2 * 2 * 2.07e9 / 1e12   # SMs x DFMA/clk x 2 flop x max clock
+# FP64 ALC screens in 64-bit fixed point: three 32 x 32 + 64-bit multiply-adds (8 lanes per clock
+# and SM sub-partition) do a term's two flops
+FX_PEAK_TFLOPS_DERIVED = 152 * 32 * 2.07e9 / 3 * 2 / 1e12
 EXP_FLOPS = 20      # FP64 flops counted per double-precision exp (measured: about 20 DFMA each)
 
 
@@ -414,7 +417,8 @@ def roofline_for(prec, w, sel_ms, traffic, method="alc"):
     """Roofline of kernels (b)+(c) for one launch over all T locations.  "frac" is always
     the method's algorithmic work (FP64-equivalent flops of the O(j)-per-candidate design:
     FMA = 2, exp = 20) per second of the launch against the peak of the pipe that does
-    it: FP64 DFMA for the FP64 kernels, FP32 FMA for the mixed screens (which carry that
+    it: FP64 DFMA for the FP64 MSPE kernel, integer multiply-adds for the fixed-point screen of
+    FP64 ALC, FP32 FMA for the mixed screens (which carry that
     work in float-float on the FP32 pipes).  For the mixed screens "issued" gives the
     second figure: the FP32 operations the float-float arithmetic actually issues, against
     the FP32 lane peak (one operation per lane-cycle)."""
@@ -424,12 +428,16 @@ def roofline_for(prec, w, sel_ms, traffic, method="alc"):
     alg = (mspe_flops_per_location if method == "mspe" else select_flops_per_location)(
         w.n0, w.n, M, w.p)
     achieved = alg * T / (sel_ms / 1e3) / 1e12
-    name = {("alc", "fp64"): "select_fp64_kernel", ("alc", "mixed"): "select_mixed_kernel",
+    name = {("alc", "fp64"): "select_mixed_kernel, fixed point", ("alc", "mixed"): "select_mixed_kernel",
             ("mspe", "fp64"): "select_mspe_kernel",
             ("mspe", "mixed"): "select_mspe_mixed_kernel"}[(method, prec)]
     out = {"kernel": name + " (kernels b+c)", "bound": "alu", "achieved": achieved,
            "unit": "TFLOP/s", "traffic": traffic, "work_per_location": alg,
            "work_unit": "FP64-equivalent flops of the O(j)-per-candidate design (FMA = 2, exp = 20)"}
+    if prec == "fp64" and method == "alc":
+        out.update(peak=FX_PEAK_TFLOPS_DERIVED, frac=achieved / FX_PEAK_TFLOPS_DERIVED,
+                   peak_source="derived integer: 152 SMs x 32 IMAD.WIDE lanes x 2.07 GHz, 3 per FMA")
+        return out
     if prec == "fp64":
         out.update(peak=FP64_PEAK_TFLOPS_DERIVED, frac=achieved / FP64_PEAK_TFLOPS_DERIVED,
                    peak_source="derived FP64: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz")

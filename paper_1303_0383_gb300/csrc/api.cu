@@ -52,11 +52,11 @@ int dev_info(DevInfo *out) {
 }
 
 int allow_smem(const void *fn, const DevInfo &di) {
-  cudaFuncAttributes fa;
+  cudaFuncAttributes fa = {};
   cudaError_t e = cudaFuncGetAttributes(&fa, fn);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(di.smem_optin - fa.sharedSizeBytes));
+  const int most = (int)(di.smem_optin - fa.sharedSizeBytes);
+  if (e == cudaSuccess && fa.maxDynamicSharedSizeBytes != most)
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   return cuda_status(e);
 }
 

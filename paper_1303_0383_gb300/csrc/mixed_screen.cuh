@@ -67,7 +67,6 @@ __device__ __forceinline__ double corr64(const double *a, const double *b, int p
 // thread's factor rows in global memory reach its own slots of a ring in shared memory a
 // few rows ahead of their use, so that the loads of the next rows are in flight while a
 // row is consumed.  Each thread waits only for its own copies (no barrier).
-constexpr int RING_A = 4;  // stages per thread, where the ring is used
 
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
