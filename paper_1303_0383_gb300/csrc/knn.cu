@@ -85,9 +85,8 @@ __device__ __forceinline__ bool key_prefix_eq(uint64_t bits, uint32_t idx, int n
   return true;
 }
 
-__device__ __forceinline__ int nthreads() { return (int)blockDim.x; }
-
 // Exclusive block scan of one value per thread; returns the prefix, *total gets the sum.
+template <int NT>
 __device__ uint32_t block_excl_scan(uint32_t v, uint32_t *warp_tmp, uint32_t *total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t inc = v;
@@ -98,25 +97,26 @@ __device__ uint32_t block_excl_scan(uint32_t v, uint32_t *warp_tmp, uint32_t *to
   if (lane == 31) warp_tmp[w] = inc;
   __syncthreads();
   if (w == 0) {
-    uint32_t s = (lane < nthreads() / 32) ? warp_tmp[lane] : 0;
+    uint32_t s = (lane < NT / 32) ? warp_tmp[lane] : 0;
     for (int o = 1; o < 32; o <<= 1) {
       uint32_t t = __shfl_up_sync(0xffffffffu, s, o);
       if (lane >= o) s += t;
     }
-    if (lane < nthreads() / 32) warp_tmp[lane] = s;  // inclusive warp totals
+    if (lane < NT / 32) warp_tmp[lane] = s;  // inclusive warp totals
   }
   __syncthreads();
   uint32_t base = (w > 0) ? warp_tmp[w - 1] : 0;
-  *total = warp_tmp[nthreads() / 32 - 1];
+  *total = warp_tmp[NT / 32 - 1];
   __syncthreads();
   return base + inc - v;
 }
 
 // Find, over hist[0..nbins), the bin where the cumulative count first reaches `rank`
 // (1-based); returns the bin and the count strictly below it.  nbins == HBINS or 256.
+template <int NT>
 __device__ void find_rank_bin(const uint32_t *hist, int nbins, uint32_t rank, uint32_t *warp_tmp,
                               int *bin_out, uint32_t *below_out) {
-  const int per = nbins / nthreads() > 0 ? nbins / nthreads() : 1;  // a power of two
+  const int per = nbins / NT > 0 ? nbins / NT : 1;  // a power of two
   const int first = threadIdx.x * per;
   uint32_t part = 0;
   // each thread's range starts at its own rotation: the lanes of a warp read different
@@ -124,7 +124,7 @@ __device__ void find_rank_bin(const uint32_t *hist, int nbins, uint32_t rank, ui
   if (first < nbins)
     for (int b = 0; b < per; b++) part += hist[first + ((b + threadIdx.x) & (per - 1))];
   uint32_t total;
-  uint32_t pre = block_excl_scan(part, warp_tmp, &total);
+  uint32_t pre = block_excl_scan<NT>(part, warp_tmp, &total);
   if (first < nbins && pre < rank && rank <= pre + part) {
     uint32_t cum = pre;
     for (int b = 0; b < per; b++) {
@@ -142,11 +142,12 @@ __device__ void find_rank_bin(const uint32_t *hist, int nbins, uint32_t rank, ui
 
 // Bitonic sort of n2 (a power of two) keys held as (hi, lo, index) words in shared memory;
 // each stage visits exactly its n2/2 compare-exchange pairs.
+template <int NT>
 __device__ void bitonic_sort(uint32_t *kh, uint32_t *kl, int32_t *idx, int n2) {
   for (int k = 2; k <= n2; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
       const int lj = __ffs(j) - 1;
-      for (int pp = threadIdx.x; pp < (n2 >> 1); pp += nthreads()) {
+      for (int pp = threadIdx.x; pp < (n2 >> 1); pp += NT) {
         const int i = ((pp >> lj) << (lj + 1)) | (pp & (j - 1));
         const int ixj = i + j;
         const uint32_t ah = kh[i], al = kl[i], bh = kh[ixj], bl = kl[ixj];
@@ -184,22 +185,23 @@ __device__ __forceinline__ double fp32_err_bound(double d, double B, int p) {
 // exact FP64 d2 of every point (recomputed in each pass, no scratch), coarse histogram of
 // float(d2), boundary resolution by radix refinement; keys into shared memory; returns
 // the count.
+template <int NT>
 __device__ int knn_exact_location(const double *__restrict__ X, int N, int p, int M,
                                   const double *xs, uint32_t *kh, uint32_t *kl, int32_t *sidx,
                                   uint32_t *hist, int cap, uint32_t *warp_tmp, int *sh_bin,
                                   uint32_t *sh_below, uint32_t *sh_count, uint32_t *pref) {
-  for (int b = threadIdx.x; b < HBINS; b += nthreads()) hist[b] = 0;
+  for (int b = threadIdx.x; b < HBINS; b += NT) hist[b] = 0;
   if (threadIdx.x == 0) *sh_count = 0;
   __syncthreads();
-  for (int i = threadIdx.x; i < N; i += nthreads())
+  for (int i = threadIdx.x; i < N; i += NT)
     atomicAdd(&hist[coarse_bin(sqdist_exact(xs, X + (size_t)i * p, p))], 1u);
   __syncthreads();
-  find_rank_bin(hist, HBINS, (uint32_t)M, warp_tmp, sh_bin, sh_below);
+  find_rank_bin<NT>(hist, HBINS, (uint32_t)M, warp_tmp, sh_bin, sh_below);
   const uint32_t bstar = (uint32_t)*sh_bin;
   const uint32_t below = *sh_below;
   const uint32_t nb = hist[bstar];
   const bool fits = below + nb <= (uint32_t)cap;
-  for (int i = threadIdx.x; i < N; i += nthreads()) {
+  for (int i = threadIdx.x; i < N; i += NT) {
     const double d2 = sqdist_exact(xs, X + (size_t)i * p, p);
     const uint32_t b = coarse_bin(d2);
     if (b < bstar || (fits && b == bstar)) put_key(kh, kl, sidx, atomicAdd(sh_count, 1u), d2, i);
@@ -209,9 +211,9 @@ __device__ int knn_exact_location(const double *__restrict__ X, int N, int p, in
     uint32_t need = (uint32_t)M - below;
     uint32_t *h256 = hist;
     for (int d = 0; d < 12; d++) {
-      for (int b = threadIdx.x; b < 256; b += nthreads()) h256[b] = 0;
+      for (int b = threadIdx.x; b < 256; b += NT) h256[b] = 0;
       __syncthreads();
-      for (int i = threadIdx.x; i < N; i += nthreads()) {
+      for (int i = threadIdx.x; i < N; i += NT) {
         const double d2 = sqdist_exact(xs, X + (size_t)i * p, p);
         if (coarse_bin(d2) != bstar) continue;
         const uint64_t bits = (uint64_t)__double_as_longlong(d2);
@@ -220,10 +222,10 @@ __device__ int knn_exact_location(const double *__restrict__ X, int N, int p, in
       }
       __syncthreads();
       const uint32_t cnt0 = *sh_count;  // stable here: no thread appends until after the scan
-      find_rank_bin(h256, 256, need, warp_tmp, sh_bin, sh_below);
+      find_rank_bin<NT>(h256, 256, need, warp_tmp, sh_bin, sh_below);
       const uint32_t dd = (uint32_t)*sh_bin, dbelow = *sh_below, deq = h256[dd];
       const bool last = cnt0 + dbelow + deq <= (uint32_t)cap;
-      for (int i = threadIdx.x; i < N; i += nthreads()) {
+      for (int i = threadIdx.x; i < N; i += NT) {
         const double d2 = sqdist_exact(xs, X + (size_t)i * p, p);
         if (coarse_bin(d2) != bstar) continue;
         const uint64_t bits = (uint64_t)__double_as_longlong(d2);
@@ -323,13 +325,13 @@ __device__ __forceinline__ int sample_rank(int N, int M) {
   return ks < ns ? ks : 0;
 }
 // hist: zeroed, HBINS bins.  Every thread returns after the same barriers.
-template <int S>
+template <int S, int NT>
 __device__ float sample_bound(const float *xf, const float *__restrict__ Xf, int N, int ks, uint32_t *hist,
                               uint32_t *warp_tmp, int *sh_bin, uint32_t *sh_below) {
-  each_point<S>(xf, Xf, N, (threadIdx.x >> 5) * 32 * KS + (threadIdx.x & 31), (nthreads() / 32) * 32 * KS,
+  each_point<S>(xf, Xf, N, (threadIdx.x >> 5) * 32 * KS + (threadIdx.x & 31), (NT / 32) * 32 * KS,
                 [&](float d2f, int) { atomicAdd(&hist[__float_as_uint(d2f) >> (31 - HBITS)], 1u); });
   __syncthreads();
-  find_rank_bin(hist, HBINS, (uint32_t)ks, warp_tmp, sh_bin, sh_below);
+  find_rank_bin<NT>(hist, HBINS, (uint32_t)ks, warp_tmp, sh_bin, sh_below);
   return __uint_as_float(((uint32_t)*sh_bin + 1u) << (31 - HBITS));
 }
 
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(KB) knn_bound_kernel(const Scan S_, int N, int
                                                        const unsigned int *__restrict__ bmax,
                                                        const int32_t *__restrict__ list,
                                                        const LocDesc *__restrict__ locs, int ldxx) {
-  constexpr int S = P ? knn_row(P) : kMaxP;
+  constexpr int S = P ? knn_row(P) : kMaxP, NT = KB;
   if (P > 0) p = P;
   const float B = __uint_as_float(*bmax);
   float s = 1.0f;
@@ -471,7 +473,7 @@ __global__ void __launch_bounds__(KB) knn_bound_kernel(const Scan S_, int N, int
     for (int b = threadIdx.x; b < HBINS; b += KB) hist[b] = 0;
     __syncthreads();
     ks = scaled ? sample_rank(N, M) : 0;
-    if (ks > 0) bound = sample_bound<S>(xf, Xf, N, ks, hist, warp_tmp, &sh_bin, &sh_below);
+    if (ks > 0) bound = sample_bound<S, NT>(xf, Xf, N, ks, hist, warp_tmp, &sh_bin, &sh_below);
   }
   if (threadIdx.x == 0) {
     float y[kMaxP], nn;
@@ -585,6 +587,7 @@ constexpr int BUCKET_CAP = 32; // largest bucket sorted in place; beyond, the bi
 // (many equal distances), leaving the keys for the bitonic sort.  The bucket bounds use
 // hist[0, nb); the permutation goes to perm (cnt entries), which may be hist + nb.
 // Every thread returns after the same barriers.
+template <int NT>
 __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32_t *sidx, int cnt,
                              int M, uint32_t *hist, int nb, uint32_t *perm, uint32_t *warp_tmp,
                              uint32_t *sh_flag, unsigned long long *sh_dmax, int32_t *out) {
@@ -593,11 +596,11 @@ __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32
     *sh_dmax = 0ull;
     *sh_flag = 0u;
   }
-  for (int b = threadIdx.x; b < nb; b += nthreads()) bound[b] = 0;
+  for (int b = threadIdx.x; b < nb; b += NT) bound[b] = 0;
   // the largest key (non-negative doubles order like their bits): a warp maximum, then one
   // shared atomic per warp
   unsigned long long wmax = 0ull;
-  for (int r = threadIdx.x; r < cnt; r += nthreads()) {
+  for (int r = threadIdx.x; r < cnt; r += NT) {
     const unsigned long long k = ((unsigned long long)kh[r] << 32) | kl[r];
     wmax = k > wmax ? k : wmax;
   }
@@ -620,10 +623,10 @@ __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32
     const int b = (int)(d2 * scale);
     return b < nb - 1 ? b : nb - 1;
   };
-  for (int r = threadIdx.x; r < cnt; r += nthreads()) atomicAdd(&bound[bucket_of(r)], 1u);
+  for (int r = threadIdx.x; r < cnt; r += NT) atomicAdd(&bound[bucket_of(r)], 1u);
   __syncthreads();
-  // exclusive scan of the counts (nb / nthreads() buckets per thread), flagging an oversized bucket
-  const int per = nb / nthreads();  // a power of two
+  // exclusive scan of the counts (nb / NT buckets per thread), flagging an oversized bucket
+  const int per = nb / NT;  // a power of two
   uint32_t part = 0;
   for (int k = 0; k < per; k++) {  // rotated start per thread: no bank conflicts
     const uint32_t c = bound[threadIdx.x * per + ((k + threadIdx.x) & (per - 1))];
@@ -631,7 +634,7 @@ __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32
     if (c > BUCKET_CAP) *sh_flag = 1u;
   }
   uint32_t total;
-  uint32_t run = block_excl_scan(part, warp_tmp, &total);
+  uint32_t run = block_excl_scan<NT>(part, warp_tmp, &total);
   for (int k = 0; k < per; k++) {
     const uint32_t c = bound[threadIdx.x * per + k];
     bound[threadIdx.x * per + k] = run;
@@ -640,12 +643,12 @@ __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32
   __syncthreads();
   if (*sh_flag) return false;
   // scatter: afterwards bound[b] is the end of bucket b (= the start of bucket b + 1)
-  for (int r = threadIdx.x; r < cnt; r += nthreads()) {
+  for (int r = threadIdx.x; r < cnt; r += NT) {
     const uint32_t at = atomicAdd(&bound[bucket_of(r)], 1u);
     if (LAGP_CHK(at, cnt, 3)) perm[at] = r;
   }
   __syncthreads();
-  for (int b = threadIdx.x; b < nb; b += nthreads()) {
+  for (int b = threadIdx.x; b < nb; b += NT) {
     const uint32_t lo = b ? bound[b - 1] : 0u, hi = bound[b];
     for (uint32_t i = lo + 1; i < hi; i++) {  // insertion by the exact key
       const uint32_t v = perm[i];
@@ -660,7 +663,7 @@ __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32
     }
   }
   __syncthreads();
-  for (int r = threadIdx.x; r < M; r += nthreads()) {
+  for (int r = threadIdx.x; r < M; r += NT) {
     const uint32_t pr = perm[r];
     out[r] = LAGP_CHK(pr, cnt, 4) ? sidx[pr] : -1;
   }
@@ -671,8 +674,8 @@ __device__ bool bucket_order(const uint32_t *kh, const uint32_t *kl, const int32
 // Batched launches pass `list` (launch position -> location), `locs` (each location's
 // candidate count and output offset) and the row stride of XX; uniform launches pass
 // nullptr and use M, t*M and t*p.
-template <int P>
-__global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const double *__restrict__ X, int N, int p,
+template <int P, int NT>
+__global__ void __launch_bounds__(NT, 4 * KB / NT) knn_kernel(const Scan S_, const double *__restrict__ X, int N, int p,
                                                  const double *__restrict__ XX, int64_t T, int M,
                                                  int32_t *__restrict__ cand,
                                                  const float *__restrict__ Xf,
@@ -711,13 +714,13 @@ __global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const dou
       xs[threadIdx.x] = x;
       xf[threadIdx.x] = __double2float_rn(x);
     }
-    for (int b = threadIdx.x; b < HBINS; b += nthreads()) hist[b] = 0;
+    for (int b = threadIdx.x; b < HBINS; b += NT) hist[b] = 0;
     if (threadIdx.x == 0) sh_count = 0;
     __syncthreads();
     // The screen's threshold thr = tau + 2E: tau the upper edge of the bin holding the M-th
     // smallest d2f in `hist` (complete up to that bin), E the FP32 error bound.
     auto set_threshold = [&]() {
-      find_rank_bin(hist, HBINS, (uint32_t)M, warp_tmp, &sh_bin, &sh_below);
+      find_rank_bin<NT>(hist, HBINS, (uint32_t)M, warp_tmp, &sh_bin, &sh_below);
       if (threadIdx.x == 0) {
         double B = Bx;
         for (int k = 0; k < p; k++) B = fmax(B, fabs(xs[k]));
@@ -738,12 +741,12 @@ __global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const dou
       some = true;
       bound = S_.bound[tt];
       const int32_t *pl = S_.list + (size_t)tt * S_.cap;
-      for (int r0 = threadIdx.x & ~31; r0 < (int)pre; r0 += KU * nthreads()) {
+      for (int r0 = threadIdx.x & ~31; r0 < (int)pre; r0 += KU * NT) {
         float d[KU];
         int id[KU];
 #pragma unroll
         for (int u = 0; u < KU; u++) {
-          const int r = r0 + u * nthreads() + (threadIdx.x & 31);
+          const int r = r0 + u * NT + (threadIdx.x & 31);
           id[u] = r < (int)pre ? pl[r] : -1;
           if (id[u] >= 0 && !LAGP_CHK(id[u], N, 2)) id[u] = -1;
         }
@@ -770,12 +773,12 @@ __global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const dou
     const int ks = sample_rank(N, M);
     if (!some && ks > 0) {
       some = true;
-      bound = sample_bound<S>(xf, Xf, N, ks, hist, warp_tmp, &sh_bin, &sh_below);
-      for (int b = threadIdx.x; b < HBINS; b += nthreads()) hist[b] = 0;
+      bound = sample_bound<S, NT>(xf, Xf, N, ks, hist, warp_tmp, &sh_bin, &sh_below);
+      for (int b = threadIdx.x; b < HBINS; b += NT) hist[b] = 0;
       __syncthreads();
       // pass 1: the points with d2f <= bound are listed (d2f bits, index) and histogrammed;
       // the list's histogram is the whole design's in every bin up to the M-th's
-      each_point<S>(xf, Xf, N, threadIdx.x, nthreads(), [&](float d2f, int i) {
+      each_point<S>(xf, Xf, N, threadIdx.x, NT, [&](float d2f, int i) {
         if (d2f <= bound) {
           const uint32_t pos = atomicAdd(&sh_count, 1u);
           if (pos < (uint32_t)cap) {
@@ -798,7 +801,7 @@ __global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const dou
           if (threadIdx.x == 0) sh_count = 0;
           __syncthreads();
           // warp-aggregated appends: one shared atomic per warp and pass
-          for (int r0 = threadIdx.x & ~31; r0 < (int)nl; r0 += nthreads()) {
+          for (int r0 = threadIdx.x & ~31; r0 < (int)nl; r0 += NT) {
             const int r = r0 + (threadIdx.x & 31);
             const bool keep = r < (int)nl && __uint_as_float(kh[r]) <= thr;
             const unsigned ball = __ballot_sync(0xffffffffu, keep);
@@ -814,21 +817,21 @@ __global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const dou
       }
       if (!listed) {  // the sample's bound missed (rare): the two full passes below
         __syncthreads();
-        for (int b = threadIdx.x; b < HBINS; b += nthreads()) hist[b] = 0;
+        for (int b = threadIdx.x; b < HBINS; b += NT) hist[b] = 0;
         if (threadIdx.x == 0) sh_count = 0;
         __syncthreads();
       }
     }
     if (!listed) {
       // pass 1: histogram of the FP32 distances of every point
-      each_point<S>(xf, Xf, N, threadIdx.x, nthreads(), [&](float d2f, int) {
+      each_point<S>(xf, Xf, N, threadIdx.x, NT, [&](float d2f, int) {
         atomicAdd(&hist[__float_as_uint(d2f) >> (31 - HBITS)], 1u);
       });
       __syncthreads();
       set_threshold();
       const float thr = sh_thr;
       // pass 2: the same FP32 distances again (bit for bit); survivors are listed first
-      each_point<S>(xf, Xf, N, threadIdx.x, nthreads(), [&](float d2f, int i) {
+      each_point<S>(xf, Xf, N, threadIdx.x, NT, [&](float d2f, int i) {
         if (d2f <= thr) {
           const uint32_t pos = atomicAdd(&sh_count, 1u);
           if (pos < (uint32_t)cap) sidx[pos] = i;
@@ -840,27 +843,27 @@ __global__ void __launch_bounds__(2 * KB, 2) knn_kernel(const Scan S_, const dou
     // then get their exact FP64 distances from the compacted list: a warp instruction of
     // the FP64 pipe serves 32 survivors instead of the few a strided pass would hold
     if (cnt <= cap)
-      for (int r = threadIdx.x; r < cnt; r += nthreads()) {
+      for (int r = threadIdx.x; r < cnt; r += NT) {
         const int32_t i = sidx[r];
         if (LAGP_CHK(i, N, 2)) put_key(kh, kl, sidx, (uint32_t)r, sqdist_exact(xs, X + (size_t)i * p, p), i);
       }
     __syncthreads();
     if (cnt > cap || cnt < M)  // too many ties at the boundary (or, defensively, too few)
-      cnt = knn_exact_location(X, N, p, M, xs, kh, kl, sidx, hist, cap, warp_tmp, &sh_bin,
+      cnt = knn_exact_location<NT>(X, N, p, M, xs, kh, kl, sidx, hist, cap, warp_tmp, &sh_bin,
                                &sh_below, &sh_count, pref);
     if (cnt > cap || cnt > perm_cap ||
-        !bucket_order(kh, kl, sidx, cnt, M, hist, nb, perm, warp_tmp, &sh_count,
+        !bucket_order<NT>(kh, kl, sidx, cnt, M, hist, nb, perm, warp_tmp, &sh_count,
                                    &sh_dmax, out)) {
       int n2 = 1;
       while (n2 < cnt) n2 <<= 1;
-      for (int i = cnt + threadIdx.x; i < n2; i += nthreads()) {
+      for (int i = cnt + threadIdx.x; i < n2; i += NT) {
         kh[i] = 0xffffffffu;
         kl[i] = 0xffffffffu;
         sidx[i] = 0x7fffffff;
       }
       __syncthreads();
-      bitonic_sort(kh, kl, sidx, n2);
-      for (int r = threadIdx.x; r < M; r += nthreads()) {
+      bitonic_sort<NT>(kh, kl, sidx, n2);
+      for (int r = threadIdx.x; r < M; r += NT) {
         const int32_t v = sidx[r];
         out[r] = LAGP_CHK(v, N, 5) ? v : -1;
       }
@@ -946,17 +949,23 @@ int knn_launch_list(const double *X, int64_t N, int32_t p, const double *XX, int
   const int cap = knn_cap(M);
   const size_t smem = knn_smem_bytes(cap);
   if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
+  // 512 threads where shared memory holds three CTAs per SM or fewer (10000 8-d locations, ncand =
+  // 2000, two CTAs: 4.15 -> 3.46 ms without the scan, 2.49 -> 2.27 with it)
+  const bool wide = knn_per_sm(smem) <= 3;
+  const int threads = wide ? 2 * KB : KB;
   const void *fn, *bfn;
   switch (p) {
 #define LAGP_KNN_CASE(P) \
-  case P: fn = (const void *)knn_kernel<P>; bfn = (const void *)knn_bound_kernel<P>; break;
+  case P: fn = wide ? (const void *)knn_kernel<P, 2 * KB> : (const void *)knn_kernel<P, KB>; \
+    bfn = (const void *)knn_bound_kernel<P>; break;
     LAGP_KNN_CASE(1)
     LAGP_KNN_CASE(2)
     LAGP_KNN_CASE(3)
     LAGP_KNN_CASE(4)
     LAGP_KNN_CASE(8)
 #undef LAGP_KNN_CASE
-    default: fn = (const void *)knn_kernel<0>; bfn = (const void *)knn_bound_kernel<0>; break;
+    default: fn = wide ? (const void *)knn_kernel<0, 2 * KB> : (const void *)knn_kernel<0, KB>;
+      bfn = (const void *)knn_bound_kernel<0>; break;
   }
   st = allow_smem(fn, di);
   if (st) return st;
@@ -1007,9 +1016,6 @@ int knn_launch_list(const double *X, int64_t N, int32_t p, const double *XX, int
       knn_scan_kernel<<<dim3(groups, (unsigned)ceil_div(tiles, part)), KB, 0, stream>>>(S, tiles, part);
       g_launches.fetch_add(2);
     }
-    // 512 threads where shared memory holds three CTAs per SM or fewer (10000 8-d locations, ncand =
-    // 2000, two CTAs: 4.15 -> 3.46 ms without the scan, 2.49 -> 2.27 with it)
-    const int threads = knn_per_sm(smem) <= 3 ? 2 * KB : KB;
     int grid = knn_grid(cnt, di.num_sms, smem);
     if (ctas_per_sm > 0) {
       const int64_t g2 = (int64_t)di.num_sms * ctas_per_sm;
