@@ -240,7 +240,9 @@ __device__ int knn_exact_location(const double *__restrict__ X, int N, int p, in
       __syncthreads();
     }
   }
-  return (int)*sh_count;
+  const int cnt = (int)*sh_count;
+  __syncthreads();  // the caller reuses the counter
+  return cnt;
 }
 
 // Floats per row of the FP32 copy of X: the dimension, padded with zeros to 1, 2, 4 or 8, so
