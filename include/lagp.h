@@ -215,8 +215,10 @@ size_t lagp_predict_batch_workspace_bytes(const lagp_design_desc *designs, int32
  * 3 <= n[t] <= 256, n[t] >= n0 of its design, n[t] <= ncand[t] <= min(N, 8192).
  * Outputs (device): mean[T], s2[T] required; var[T], status[T] optional; idx, optional,
  * holds sum(n) indices, location t's n[t] at offset n[0] + ... + n[t-1].
- * flags: LAGP_BATCH_TUNE and/or LAGP_BATCH_GRAPH (see above; graphs are cached per
- * signature and buffer set, and the per-location tables are copied in before each replay).
+ * flags: LAGP_BATCH_TUNE and/or LAGP_BATCH_GRAPH (see above; the 64 graphs used last are
+ * kept; one is replayed, after the per-location tables are copied in, where buffers, T and
+ * the sizes that lay out the launches are the same: the largest n and ncand, the sums of n and
+ * of ncand, and each design's location count and largest ncand).
  * The call enqueues on `stream`; with LAGP_BATCH_TUNE on a new signature it synchronises. */
 int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t ndesigns, const double *XX,
                            int32_t ldxx, int64_t T, const int32_t *design_of, const int32_t *n,

@@ -9,15 +9,17 @@
 //                     timing the candidates on the first batch of each signature (method,
 //                     precision, dimensions present, n and M buckets, T bucket); the choice
 //                     is cached for the process;
-//   LAGP_BATCH_GRAPH  the launches are captured into a CUDA graph the first time a batch
-//                     signature and buffer set is seen, and the graph is replayed afterwards
-//                     (the tables are copied in before each replay).
+//   LAGP_BATCH_GRAPH  the launches are captured into a CUDA graph the first time a set of
+//                     sizes and buffers is seen (batch_graph_key), and the graph is replayed
+//                     afterwards (the tables are copied in before each replay).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <string.h>
 
 #include <algorithm>
+#include <list>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <numeric>
 #include <string>
@@ -29,23 +31,9 @@
 namespace lagp {
 namespace {
 
-struct Layout {
-  size_t designs, locs, order, lists, cand, scratch, total;
-  size_t knn_ws, sel_ws;
-};
-
-struct Plan {
-  std::vector<BatchDesign> designs;
-  std::vector<LocDesc> locs;
-  std::vector<int32_t> order, lists, list_off, list_cnt;
-  int32_t nmax = 0, pmax = 0, Mmax = 0;
-  std::vector<int32_t> Mmax_d;
-  int64_t cand_total = 0, idx_total = 0, Nmax = 0;
-};
-
 int validate_and_plan(const lagp_design_desc *designs, int32_t nd, int64_t T, const int32_t *design_of,
                       const int32_t *n, const int32_t *ncand, int32_t method, int32_t precision,
-                      Plan *P) {
+                      BatchPlan *P) {
   if (nd < 1 || T < 0 || (T > 0 && (!design_of || !n || !ncand)) || !designs) return LAGP_ERR_INVALID_ARG;
   if (method != LAGP_ALC && method != LAGP_MSPE && method != LAGP_NN) return LAGP_ERR_INVALID_ARG;
   if (precision != LAGP_FP64 && precision != LAGP_MIXED) return LAGP_ERR_INVALID_ARG;
@@ -97,7 +85,7 @@ int validate_and_plan(const lagp_design_desc *designs, int32_t nd, int64_t T, co
   return LAGP_OK;
 }
 
-BatchLaunch make_launch(const Plan &P, int32_t method, int32_t precision, int64_t T,
+BatchLaunch make_launch(const BatchPlan &P, int32_t method, int32_t precision, int64_t T,
                         const double *XX, int32_t ldxx, double *mean, double *s2, double *var,
                         int32_t *idx, int8_t *status, int ctas) {
   BatchLaunch b;
@@ -113,16 +101,15 @@ BatchLaunch make_launch(const Plan &P, int32_t method, int32_t precision, int64_
   b.nmax = P.nmax;
   b.pmax = P.pmax;
   b.Mmax = P.Mmax;
-  b.gmin = INFINITY;
-  for (const auto &d : P.designs) b.gmin = std::min(b.gmin, d.g);
+  b.gmin = P.gmin();
   b.mean = mean; b.s2 = s2; b.var = var; b.idx = idx; b.status = status;
   b.idx_total = P.idx_total;
   b.ctas_per_sm = ctas;
   return b;
 }
 
-Layout layout_of(const Plan &P, int32_t method, int32_t precision, int64_t T, int num_sms) {
-  Layout L;
+BatchLayout layout_of(const BatchPlan &P, int32_t method, int32_t precision, int64_t T, int num_sms) {
+  BatchLayout L;
   L.designs = 0;
   L.locs = align_up(L.designs + P.designs.size() * sizeof(BatchDesign), 256);
   L.order = align_up(L.locs + (size_t)T * sizeof(LocDesc), 256);
@@ -144,7 +131,7 @@ struct TuneChoice {
 std::mutex g_tune_mu;
 std::map<std::string, TuneChoice> g_tune;
 
-std::string signature(const Plan &P, int32_t method, int32_t precision, int64_t T) {
+std::string signature(const BatchPlan &P, int32_t method, int32_t precision, int64_t T) {
   std::string k = std::to_string(method) + "/" + std::to_string(precision) + "/p";
   bool seen[kMaxP + 1] = {false};
   for (const auto &d : P.designs) seen[d.p] = true;
@@ -157,16 +144,46 @@ std::string signature(const Plan &P, int32_t method, int32_t precision, int64_t 
   return k;
 }
 
-// ---- graph cache: one instantiated graph per (signature, buffers, launch shape)
+// ---- graph cache: one instantiated graph per batch_graph_key, the kGraphs used last
+constexpr size_t kGraphs = 64;
 std::mutex g_graph_mu;
 // An instantiated graph and the number of kernels it launches (counted at capture, where
 // the launches are recorded but do not run; added to the launch counter at each replay).
+// A thread that is about to launch an entry keeps it alive; a graph destroyed while it runs is
+// freed when it ends.  The handle goes with its context (cudaDeviceReset).
 struct GraphEntry {
-  cudaGraphExec_t exec;
-  int64_t kernels;
+  cudaGraphExec_t exec = nullptr;
+  int64_t kernels = 0;
+  unsigned long long context = 0;
+  ~GraphEntry() {
+    unsigned long long id = 0;
+    if (exec && current_context_id(&id) == LAGP_OK && id == context) cudaGraphExecDestroy(exec);
+  }
 };
-std::map<std::string, GraphEntry> g_graphs;
+using GraphList = std::list<std::pair<std::string, std::shared_ptr<GraphEntry>>>;
+GraphList &graphs() {  // the last used first; kept until the process exits, after the CUDA runtime
+  static GraphList *l = new GraphList;
+  return *l;
+}
 
+std::shared_ptr<GraphEntry> graph_find(const std::string &k) {
+  std::lock_guard<std::mutex> lk(g_graph_mu);
+  GraphList &l = graphs();
+  for (auto it = l.begin(); it != l.end(); ++it)
+    if (it->first == k) {
+      l.splice(l.begin(), l, it);
+      return it->second;
+    }
+  return nullptr;
+}
+
+void graph_keep(const std::string &k, std::shared_ptr<GraphEntry> g) {
+  std::lock_guard<std::mutex> lk(g_graph_mu);
+  graphs().emplace_front(k, std::move(g));
+  if (graphs().size() > kGraphs) graphs().pop_back();
+}
+
+std::mutex g_capture_mu;  // one capture at a time: they share the stream
 // One non-blocking stream per device for graph capture (created on first use).
 cudaStream_t capture_stream(int device) {
   static std::mutex mu;
@@ -181,7 +198,7 @@ cudaStream_t capture_stream(int device) {
 }  // namespace
 
 // The launches of one batch (kernel (a) per design, then kernels (b)+(c)).
-static int launch_all(const Plan &P, const Layout &L, char *w, const double *XX, int32_t ldxx,
+static int launch_all(const BatchPlan &P, const BatchLayout &L, char *w, const double *XX, int32_t ldxx,
                       int64_t T, int32_t method, int32_t precision, double *mean, double *s2,
                       double *var, int32_t *idx, int8_t *status, int knn_ctas, int sel_ctas,
                       cudaStream_t stream) {
@@ -216,7 +233,7 @@ extern "C" size_t lagp_predict_batch_workspace_bytes(const lagp_design_desc *des
                                                      int64_t T, const int32_t *design_of,
                                                      const int32_t *n, const int32_t *ncand,
                                                      int32_t method, int32_t precision) {
-  Plan P;
+  BatchPlan P;
   if (validate_and_plan(designs, ndesigns, T, design_of, n, ncand, method, precision, &P)) return 0;
   DevInfo di;
   if (dev_info(&di)) return 0;
@@ -230,7 +247,7 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
                                       double *mean, double *s2, double *var, int32_t *idx,
                                       int8_t *status, uint32_t flags, void *workspace,
                                       size_t workspace_bytes, void *stream_) {
-  Plan P;
+  BatchPlan P;
   int st = validate_and_plan(designs, ndesigns, T, design_of, n, ncand, method, precision, &P);
   if (st) return st;
   if (T == 0) return LAGP_OK;
@@ -239,7 +256,7 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
   DevInfo di;
   st = dev_info(&di);
   if (st) return st;
-  const Layout L = layout_of(P, method, precision, T, di.num_sms);
+  const BatchLayout L = layout_of(P, method, precision, T, di.num_sms);
   if (workspace_bytes < L.total) return LAGP_ERR_INVALID_ARG;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   char *w = static_cast<char *>(workspace);
@@ -298,27 +315,17 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
     return LAGP_OK;  // every timed run produced the outputs; they do not depend on the shape
   }
   if (flags & LAGP_BATCH_GRAPH) {
-    char key[512];
-    snprintf(key, sizeof key, "%s|%p|%p|%d|%p|%p|%p|%p|%p|%d|%d|%zu", sig.c_str(), (void *)w,
-             (const void *)XX, ldxx, (void *)mean, (void *)s2, (void *)var, (void *)idx,
-             (void *)status, knn_ctas, sel_ctas, (size_t)T);
-    std::string k(key);
-    for (const auto &d : P.designs) {
-      char dk[96];
-      snprintf(dk, sizeof dk, "|%p,%p,%lld", (const void *)d.X, (const void *)d.Z, (long long)d.N);
-      k += dk;
-    }
-    cudaGraphExec_t exec = nullptr;
-    int64_t kernels = 0;
-    {
-      std::lock_guard<std::mutex> lk(g_graph_mu);
-      auto it = g_graphs.find(k);
-      if (it != g_graphs.end()) {
-        exec = it->second.exec;
-        kernels = it->second.kernels;
-      }
-    }
-    if (!exec) {
+    BatchCall C;
+    memset(&C, 0, sizeof C);
+    C.workspace = w; C.workspace_bytes = workspace_bytes;
+    C.XX = XX; C.ldxx = ldxx; C.T = T; C.method = method; C.precision = precision;
+    C.mean = mean; C.s2 = s2; C.var = var; C.idx = idx; C.status = status;
+    C.knn_ctas = knn_ctas; C.sel_ctas = sel_ctas;
+    st = current_context_id(&C.context);
+    if (st) return st;
+    const std::string k = batch_graph_key(P, L, C);
+    std::shared_ptr<GraphEntry> g = graph_find(k);
+    if (!g) {
       // Capture on a library-owned stream (the legacy default stream cannot be captured);
       // the graph is then launched on the caller's stream, after the table copies.
       st = select_prepare();
@@ -328,25 +335,27 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
       if (st) return st;
       cudaStream_t cap = capture_stream(di.device);
       if (!cap) return LAGP_ERR_CUDA;
+      g = std::make_shared<GraphEntry>();
+      g->context = C.context;
       cudaGraph_t graph;
+      std::lock_guard<std::mutex> lk(g_capture_mu);
       e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
       if (e != cudaSuccess) return cuda_status(e);
       const int64_t before = g_launches.load();
       st = launch_all(P, L, w, XX, ldxx, T, method, precision, mean, s2, var, idx, status,
                       knn_ctas, sel_ctas, cap);
-      kernels = g_launches.load() - before;
-      g_launches.fetch_sub(kernels);  // recorded, not run
+      g->kernels = g_launches.load() - before;
+      g_launches.fetch_sub(g->kernels);  // recorded, not run
       e = cudaStreamEndCapture(cap, &graph);
       if (st) return st;
       if (e != cudaSuccess) return cuda_status(e);
-      e = cudaGraphInstantiate(&exec, graph, 0);
+      e = cudaGraphInstantiate(&g->exec, graph, 0);
       cudaGraphDestroy(graph);
       if (e != cudaSuccess) return cuda_status(e);
-      std::lock_guard<std::mutex> lk(g_graph_mu);
-      g_graphs[k] = GraphEntry{exec, kernels};
+      graph_keep(k, g);
     }
-    e = cudaGraphLaunch(exec, stream);
-    if (e == cudaSuccess) g_launches.fetch_add(kernels);
+    e = cudaGraphLaunch(g->exec, stream);
+    if (e == cudaSuccess) g_launches.fetch_add(g->kernels);
     return cuda_status(e);
   }
   return launch_all(P, L, w, XX, ldxx, T, method, precision, mean, s2, var, idx, status, knn_ctas,

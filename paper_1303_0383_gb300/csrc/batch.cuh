@@ -8,21 +8,9 @@
 
 #include <stdint.h>
 
+#include "batch_plan.h"
+
 namespace lagp {
-
-struct BatchDesign {
-  const double *X;  // N x p, device
-  const double *Z;  // N, device
-  int64_t N;
-  int32_t p, n0;
-  double theta, g;
-};
-
-struct LocDesc {
-  int32_t design, n, M, pad;
-  int64_t cand_off;  // offset of this location's candidate list
-  int64_t idx_off;   // offset of this location's selected indices (in the idx output)
-};
 
 // Launch-wide view of the tables (device pointers) plus the uniform fallback values.
 struct BatchView {
