@@ -301,18 +301,55 @@ __device__ __forceinline__ float sqdist_f32(const float *xf, const float *__rest
 
 // Visits the points i = first, first + stride, ... < N: the FP32 distances of KU points are
 // formed -- their loads in flight together -- before f(d2f, i) uses any of them (one point
-// at a time, each pass was bound by the L2 latency of its dependent loads).
+// at a time, each pass was bound by the L2 latency of its dependent loads).  first is the
+// thread's lane past a multiple of 32, stride a multiple of 32: a warp visits 32 neighbours.
+// Rows of 8: a lane that loaded its own point's row would touch every line of 32 rows twice; the
+// warp loads them as they lie instead, lane l the half row l & 1 of point l / 2, the even lanes start
+// the sum and the odd ones end it (the same operations in the same order), and the even lanes
+// take over half of the points.  GB300, 3000 8-d locations over 100000 points far from the origin
+// (not scanned), ncand = 1000: 1.00 ms a row per lane -> 0.87 (a dimension-major copy: 0.83; the
+// lists of the scan want rows); 20000 points: 0.36 -> 0.35.
 constexpr int KU = 4;
 template <int S, typename F>
 __device__ __forceinline__ void each_point(const float *xf, const float *__restrict__ Xf, int N,
                                            int first, int stride, F f) {
   int i = first;
-  for (; i + (KU - 1) * stride < N; i += KU * stride) {
-    float d[KU];
+  if constexpr (S == 8) {
+    const int lane = threadIdx.x & 31, odd = lane & 1;
+    const float x0 = xf[4 * odd], x1 = xf[4 * odd + 1], x2 = xf[4 * odd + 2], x3 = xf[4 * odd + 3];
+    // the half row's sum, on top of a
+    auto half = [&](float a, const float4 &v) {
+      const float d0 = __fsub_rn(x0, v.x), d1 = __fsub_rn(x1, v.y), d2 = __fsub_rn(x2, v.z), d3 = __fsub_rn(x3, v.w);
+      return __fmaf_rn(d3, d3, __fmaf_rn(d2, d2, __fmaf_rn(d1, d1, __fmaf_rn(d0, d0, a))));
+    };
+    const int mine = odd ? lane >> 1 : 16 + (lane >> 1);
+    for (; i - lane + (KU - 1) * stride + 31 < N; i += KU * stride) {
+      float4 v[KU][2];
+      float d[KU];
 #pragma unroll
-    for (int u = 0; u < KU; u++) d[u] = sqdist_f32<S>(xf, Xf, i + u * stride);
+      for (int u = 0; u < KU; u++) {
+        const float4 *r = reinterpret_cast<const float4 *>(Xf + (size_t)(i - lane + u * stride) * S) + lane;
+        v[u][0] = r[0];
+        v[u][1] = r[32];
+      }
 #pragma unroll
-    for (int u = 0; u < KU; u++) f(d[u], i + u * stride);
+      for (int u = 0; u < KU; u++) {
+        const float a = half(__shfl_up_sync(0xffffffffu, half(0.0f, v[u][0]), 1), v[u][0]);  // points 0 .. 15
+        const float b = half(__shfl_up_sync(0xffffffffu, half(0.0f, v[u][1]), 1), v[u][1]);  // 16 .. 31
+        const float o = __shfl_down_sync(0xffffffffu, b, 1);
+        d[u] = odd ? a : o;
+      }
+#pragma unroll
+      for (int u = 0; u < KU; u++) f(d[u], i - lane + u * stride + mine);
+    }
+  } else {
+    for (; i + (KU - 1) * stride < N; i += KU * stride) {
+      float d[KU];
+#pragma unroll
+      for (int u = 0; u < KU; u++) d[u] = sqdist_f32<S>(xf, Xf, i + u * stride);
+#pragma unroll
+      for (int u = 0; u < KU; u++) f(d[u], i + u * stride);
+    }
   }
   for (; i < N; i += stride) f(sqdist_f32<S>(xf, Xf, i), i);
 }
@@ -516,6 +553,11 @@ __global__ void __launch_bounds__(KB) knn_scan_kernel(const Scan S_, int tiles, 
     b1[c] = x[q + 4];
     th[c] = *reinterpret_cast<const float2 *>(S_.thr + loc0 + 8 * c + 2 * q);
   }
+  // nothing to do where none of the 64 is to be scanned (each warp holds all their thresholds)
+  bool any = false;
+#pragma unroll
+  for (int c = 0; c < kScanLocs / 8; c++) any = any || th[c].x > -INFINITY || th[c].y > -INFINITY;
+  if (!__any_sync(0xffffffffu, any)) return;
   const int first = blockIdx.y * part, last = min(first + part, tiles);
   for (int base = first; base < last; base += kScanTiles) {
     const int end = min(kScanTiles, last - base);
@@ -737,7 +779,8 @@ __global__ void __launch_bounds__(NT, 4 * KB / NT) knn_kernel(const Scan S_, con
     bool listed = false;
     float bound = 0.0f;
     bool some = false;  // (d2f, index) of the points with d2f <= bound are listed
-    const uint32_t pre = S_.cnt ? S_.cnt[tt] : 0u;
+    const bool scanned = S_.cnt && S_.thr[tt] > -INFINITY;
+    const uint32_t pre = scanned ? S_.cnt[tt] : 0u;
     if (pre >= (uint32_t)M && pre <= (uint32_t)S_.cap) {
       // the scan listed every point that can have d2f <= bound (and a few more)
       some = true;
@@ -772,12 +815,16 @@ __global__ void __launch_bounds__(NT, 4 * KB / NT) knn_kernel(const Scan S_, con
         }
       }
     }
-    const int ks = sample_rank(N, M);
+    // (a scan that listed fewer than M has shown that the sample's bound missed: two full passes)
+    const int ks = scanned && pre < (uint32_t)M ? 0 : sample_rank(N, M);
     if (!some && ks > 0) {
       some = true;
-      bound = sample_bound<S, NT>(xf, Xf, N, ks, hist, warp_tmp, &sh_bin, &sh_below);
-      for (int b = threadIdx.x; b < HBINS; b += NT) hist[b] = 0;
-      __syncthreads();
+      bound = S_.cnt ? S_.bound[tt] : INFINITY;  // the kernel before the scan has it
+      if (!(bound < INFINITY)) {
+        bound = sample_bound<S, NT>(xf, Xf, N, ks, hist, warp_tmp, &sh_bin, &sh_below);
+        for (int b = threadIdx.x; b < HBINS; b += NT) hist[b] = 0;
+        __syncthreads();
+      }
       // pass 1: the points with d2f <= bound are listed (d2f bits, index) and histogrammed;
       // the list's histogram is the whole design's in every bin up to the M-th's
       each_point<S>(xf, Xf, N, threadIdx.x, NT, [&](float d2f, int i) {
