@@ -180,7 +180,7 @@ int lagp_design_destroy(lagp_design *d) {
 size_t lagp_knn_workspace_bytes(int64_t N, int64_t T, int32_t ncand) {
   DevInfo di;
   if (dev_info(&di)) return 0;
-  return knn_workspace_bytes(N, T, ncand, di.num_sms);
+  return knn_asked_bytes(N, T, ncand);
 }
 
 int lagp_knn_dev(const double *X, int64_t N, int32_t p, const double *XX, int64_t T,
@@ -299,7 +299,7 @@ size_t lagp_predict_workspace_bytes(int64_t N, int64_t T, int32_t p, int32_t n, 
   DevInfo di;
   if (dev_info(&di)) return 0;
   size_t cand = align_up((size_t)(T > 0 ? T : 0) * (size_t)ncand * sizeof(int32_t), 256);
-  size_t a = knn_workspace_bytes(N, T, ncand, di.num_sms);
+  size_t a = knn_asked_bytes(N, T, ncand);
   size_t b = select_workspace_bytes(T, p, n, ncand, method, precision, di.num_sms);
   return cand + (a > b ? a : b);
 }

@@ -116,7 +116,7 @@ BatchLayout layout_of(const BatchPlan &P, int32_t method, int32_t precision, int
   L.lists = align_up(L.order + (size_t)T * sizeof(int32_t), 256);
   L.cand = align_up(L.lists + (size_t)T * sizeof(int32_t), 256);
   L.scratch = align_up(L.cand + (size_t)P.cand_total * sizeof(int32_t), 256);
-  L.knn_ws = knn_workspace_bytes(P.Nmax, T, P.Mmax, num_sms);
+  L.knn_ws = knn_asked_bytes(P.Nmax, T, P.Mmax);
   BatchLaunch b = make_launch(P, method, precision, T, nullptr, 0, nullptr, nullptr, nullptr,
                               nullptr, nullptr, select_max_ctas(method, precision));
   L.sel_ws = select_batch_workspace_bytes(b, num_sms);

@@ -8,6 +8,7 @@
 
 #include "lagp.h"
 #include "batch.cuh"
+#include "sizes.h"
 
 namespace lagp {
 
@@ -17,9 +18,6 @@ constexpr int kMaxN = 256;       // local design size n
 constexpr int kMaxCand = 8192;   // candidate count
 
 extern std::atomic<int64_t> g_launches;
-
-inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
-inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // Device properties of the current device, cached per device ordinal.
 struct DevInfo {
@@ -35,7 +33,6 @@ int dev_info(DevInfo *out);
 int allow_smem(const void *fn, const DevInfo &di);
 
 // Kernel (a): candidate sets.
-size_t knn_workspace_bytes(int64_t N, int64_t T, int32_t ncand, int num_sms);
 int knn_launch(const double *X, int64_t N, int32_t p, const double *XX, int64_t T, int32_t ncand,
                int32_t *cand, void *ws, size_t ws_bytes, cudaStream_t stream);
 int knn_launch_list(const double *X, int64_t N, int32_t p, const double *XX, int64_t nloc,

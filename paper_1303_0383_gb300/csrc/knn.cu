@@ -398,7 +398,6 @@ struct Scan {
   uint32_t *xfrag;    // the locations: 8 words (16 halves) each
   float *thr;         // threshold - |x|^2; -inf: not scanned
 };
-constexpr int kScanLocs = 64;    // locations of a CTA (8 column tiles)
 constexpr int kScanTiles = 128;  // row tiles (16 points) between two extractions
 
 // The 16 values of a point (y = its scaled coordinates) or, x = true, of a location.
@@ -921,12 +920,6 @@ __global__ void __launch_bounds__(NT, 4 * KB / NT) knn_kernel(const Scan S_, con
   }
 }
 
-int knn_cap(int M) {
-  int cap = 2048;
-  while (cap < 2 * M && cap < 16384) cap <<= 1;
-  return cap;
-}
-
 size_t knn_smem_bytes(int cap) {
   return (size_t)cap * (4 + 4 + 4) + HBINS * 4 + (knn_own_perm(cap) ? (size_t)cap * 4 : 0);
 }
@@ -944,43 +937,13 @@ int knn_grid(int64_t T, int num_sms, size_t smem) {
 
 int knn_check_take(CheckRec *out) { return check_take_here(out); }
 
-// Scratch layout: [bmax (256 B)] [Xf: N rows of up to kMaxP floats], then, for the scan, the
-// design's operands and a wave of locations: [counts, bounds, thresholds, operands, lists].
-struct ScanLayout {
-  int cap, wave;  // list entries per location, locations per wave
-  size_t frag, locs, total;
-};
-constexpr size_t kScanListBytes = 128u << 20;
-
-static size_t knn_base_bytes(int64_t N) { return 256 + align_up((size_t)N * kMaxP * sizeof(float), 256); }
-
-static size_t scan_loc_bytes(int cap) { return 44 + (size_t)cap * sizeof(int32_t); }
-
-static ScanLayout scan_layout(int64_t N, int64_t T, int32_t M) {
-  ScanLayout L;
-  L.cap = knn_cap(M) + knn_cap(M) / 2;
-  int64_t w = (int64_t)(kScanListBytes / (L.cap * sizeof(int32_t)));
-  if (w < 512) w = 512;
-  if (w > T) w = T;
-  L.wave = (int)(ceil_div(w, kScanLocs) * kScanLocs);
-  L.frag = knn_base_bytes(N);
-  L.locs = L.frag + align_up((size_t)ceil_div(N, 16) * 512, 256);
-  L.total = L.locs + 256 + L.wave * scan_loc_bytes(L.cap);
-  return L;
-}
-
 // The scan is three launches (bounds, scan, lists to candidates) instead of one, for designs
 // large enough that pass 1 is most of a location's work.  GB300, whole search, per-location
 // passes -> scan: N = 40000 as above, 100 locations of 500 among 100000 70 -> 58 us; N = 16384, 2-d,
 // ncand = 1000: one location 35 -> 41 us, 100 44 -> 54, 3000 183 -> 194.
 // The last condition: distances that the scan's precision separates, if the points fill a box.
 static bool scan_pays(int64_t N, int32_t M, int p) {
-  return N >= 32768 && N >= 8 * (int64_t)M && pow(1.5 * M / N, 2.0 / p) >= (p <= 4 ? 4e-4 : 3e-2);
-}
-
-size_t knn_workspace_bytes(int64_t N, int64_t T, int32_t ncand, int num_sms) {
-  (void)num_sms;
-  return N >= 32768 && T > 0 ? scan_layout(N, T, ncand).total : knn_base_bytes(N);
+  return N >= kScanMinN && N >= 8 * (int64_t)M && pow(1.5 * M / N, 2.0 / p) >= (p <= 4 ? 4e-4 : 3e-2);
 }
 
 // Launch kernel (a) over nloc locations of one design.  Uniform launches: list == nullptr,
@@ -1029,26 +992,27 @@ int knn_launch_list(const double *X, int64_t N, int32_t p, const double *XX, int
   knn_prep_kernel<<<pblocks, KB, 0, stream>>>(X, N, p, Xf, bmax);
   g_launches.fetch_add(1);
   const int Ni = (int)N;
-  ScanLayout L = scan_layout(N, nloc, M);
-  // (a batch's workspace is sized for its largest N, M and T, whose wave may be another)
-  const int64_t room = ws_bytes < L.locs + 256 ? 0 : (int64_t)((ws_bytes - L.locs - 256) / scan_loc_bytes(L.cap));
-  if (room < L.wave) L.wave = (int)(room / kScanLocs * kScanLocs);
-  const bool scan = scan_pays(N, M, p) && L.wave > 0;
-  const int64_t waves = scan ? ceil_div(nloc, L.wave) : 1;
-  const int64_t share = ceil_div(ceil_div(nloc, waves), kScanLocs) * kScanLocs;  // <= L.wave
+  // the scan's part of the workspace: its operands, then as many locations as there is room for
+  // (a batch's is sized for its largest N, M and T)
+  const size_t frag_off = knn_base_bytes(N), loc_off = frag_off + scan_frag_bytes(N);
+  const int lcap = scan_cap(M);
+  const int64_t wave = ws_bytes < loc_off + 256 ? 0 : scan_wave(ws_bytes - loc_off - 256, nloc, M);
+  const bool scan = scan_pays(N, M, p) && wave > 0;
+  const int64_t waves = scan ? ceil_div(nloc, wave) : 1;
+  const int64_t share = ceil_div(ceil_div(nloc, waves), kScanLocs) * kScanLocs;  // <= wave
   for (int64_t first = 0; first < nloc; first += share) {
     int64_t cnt = waves == 1 || nloc - first < share ? nloc - first : share;
     Scan S;
     S.first = first;
     S.cnt = nullptr;
     if (scan) {
-      S.cnt = reinterpret_cast<uint32_t *>(w + L.locs);
-      S.bound = reinterpret_cast<float *>(S.cnt + L.wave);
-      S.thr = S.bound + L.wave;
-      S.xfrag = reinterpret_cast<uint32_t *>(S.thr + L.wave);
-      S.list = reinterpret_cast<int32_t *>(w + L.locs + align_up((size_t)L.wave * 44, 256));
-      S.frag = reinterpret_cast<uint4 *>(w + L.frag);
-      S.cap = L.cap;
+      S.cnt = reinterpret_cast<uint32_t *>(w + loc_off);
+      S.bound = reinterpret_cast<float *>(S.cnt + wave);
+      S.thr = S.bound + wave;
+      S.xfrag = reinterpret_cast<uint32_t *>(S.thr + wave);
+      S.list = reinterpret_cast<int32_t *>(w + loc_off + align_up((size_t)wave * 44, 256));
+      S.frag = reinterpret_cast<uint4 *>(w + frag_off);
+      S.cap = lcap;
       int c = (int)cnt, npad = (int)(ceil_div(cnt, kScanLocs) * kScanLocs);
       const int tiles = (int)ceil_div(N, 16);
       const int conv = first ? 0 : (int)std::min<int64_t>(ceil_div(16 * (int64_t)tiles, KB), 4 * di.num_sms);

@@ -40,8 +40,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kMaxCL = 8;          // CTAs per cluster in the cluster form
-constexpr int kScrThreads = 512;   // threads per SM: CTAs of 128, 256 or 512 threads, 128 registers each
 
 // A location's formats (fx.cuh), and what they are found from.
 struct FxFormat {
@@ -562,10 +560,6 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
   }
 }
 
-// Candidate pairs of one CTA slot: M candidates over CL CTAs, padded to 32 pairs (so the
-// shared-memory rows after the Mpad = 2 Qpad flag bytes start 16-byte aligned).
-int mix_qpad(int M, int CL) { return (int)align_up((size_t)ceil_div(ceil_div(M, 2), CL), 32); }
-
 // The kernel instance of a launch: threads per CTA and CTAs per location (CL > 1: the cluster
 // form, 256 threads).
 struct MixVariant {
@@ -619,11 +613,9 @@ int mix_cluster_size() {
   return e == 1 || e == 2 || e == 4 || e == 8 ? e : 1;
 }
 
-// Threads per CTA: one candidate pair per thread where 256, 512 or 1024 threads cover them.
 MixVariant mix_variant(int M, int CL, bool fixed) {
   if (CL > 1) return MixVariant{256, 2, CL, false};
-  const int Qpad = mix_qpad(M, 1);
-    return MixVariant{Qpad <= 256 ? 128 : Qpad <= 512 ? 256 : 512, Qpad <= 128 ? 1 : 2, 1, fixed};
+  return MixVariant{mix_threads(M), mix_qpad(M, 1) <= 128 ? 1 : 2, 1, fixed};
 }
 
 // Records and dynamic shared memory of a launch whose largest location has Qpad pairs and n
@@ -684,36 +676,6 @@ int mix_cluster_grid(int64_t T, MixVariant v, size_t smem, const DevInfo &di, in
   c = c < (T > 0 ? T : 1) ? c : (T > 0 ? T : 1);
   *G = (int)(c * v.CL);
   return LAGP_OK;
-}
-
-struct MixLayout {
-  size_t u, xr, a, idx, pred, total;
-};
-
-// [queue | re-score counter | U | Xr | A | design indices | kernel (c) workspace]
-MixLayout mix_layout(int G, int p, int n, int Qpad, int64_t T, int64_t idx_total, int num_sms) {
-  MixLayout L;
-  L.u = align_up((size_t)G * n * Qpad * sizeof(int4), 256);
-  L.xr = align_up((size_t)G * p * Qpad * sizeof(int4), 256);
-  L.a = align_up((size_t)G * n * (n + 2) * sizeof(double), 256);
-  L.idx = align_up((size_t)idx_total * sizeof(int32_t), 256);
-  L.pred = predict_fp64_workspace_bytes(T, n, num_sms);
-  L.total = 256 + 256 + L.u + L.xr + L.a + L.idx + L.pred;
-  return L;
-}
-
-// The workspace of a uniform launch covers every instance and cluster size (the grid has
-// at most min(resident CTAs per SM x SMs, CL x T) CTAs).
-size_t mix_uniform_bytes(int64_t T, int p, int n, int M, int num_sms) {
-  size_t best = 0;
-  for (int CL = 1; CL <= kMaxCL; CL *= 2) {
-    int64_t G = (int64_t)num_sms * mix_minb(mix_variant(M, CL, false));
-    const int64_t cap = (int64_t)CL * (T > 0 ? T : 1);
-    G = G < cap ? G : cap;
-    const size_t b = mix_layout((int)G, p, n, mix_qpad(M, CL), T, T * n, num_sms).total;
-    best = b > best ? b : best;
-  }
-  return best;
 }
 
 // The screen, then kernel (c) on the designs it selected.
@@ -783,7 +745,7 @@ int mix_batch_grid(const BatchLaunch &b, int num_sms) {
 int select_mixed_check_take(CheckRec *out) { return check_take_here(out); }
 
 size_t select_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms) {
-  return mix_uniform_bytes(T, p, n, ncand, num_sms);
+  return mix_asked_bytes(T, p, n, ncand, T * n, predict_fp64_workspace_bytes(T, n, num_sms), num_sms, true);
 }
 
 int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -803,7 +765,10 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
     st = mix_cluster_grid(a.T, v, smem, di, &G);
     if (st) return st;
   }
-  const MixLayout L = mix_layout(G, a.p, a.n, Qpad, a.T, a.T * a.n, di.num_sms);
+  const size_t pred = predict_fp64_workspace_bytes(a.T, a.n, di.num_sms);
+  if (v.CL == 1) G = mix_fit(G, ws_bytes, a.p, a.n, Qpad, a.T * a.n, pred, di.num_sms);
+  if (G < 1) return LAGP_ERR_INVALID_ARG;
+  const MixLayout L = mix_layout(G, a.p, a.n, Qpad, a.T * a.n, pred);
   if (ws_bytes < L.total) return LAGP_ERR_INVALID_ARG;
   MixParams P;
   P.X = a.X; P.Z = a.Z; P.N = a.N; P.p = a.p; P.XX = a.XX; P.T = a.T; P.cand = a.cand;
@@ -820,7 +785,8 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
 size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b) {
   DevInfo di;
   const int sms = dev_info(&di) == LAGP_OK ? di.num_sms : 152;
-  return mix_layout(mix_batch_grid(b, sms), b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.T, b.idx_total, sms).total;
+  return mix_asked_bytes(b.T, b.pmax, b.nmax, b.Mmax, b.idx_total, predict_fp64_workspace_bytes(b.T, b.nmax, sms), sms,
+                         false);
 }
 
 // (Locations grouped by candidate count, one launch of a fitting instance each, measured slower:
@@ -831,9 +797,11 @@ int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, c
   if (st) return st;
   st = exp_table_upload();  // this translation unit's copy of the exp constants
   if (st) return st;
-  const int G = mix_batch_grid(b, di.num_sms), Qpad = mix_qpad(b.Mmax, 1);
-  const MixLayout L = mix_layout(G, b.pmax, b.nmax, Qpad, b.T, b.idx_total, di.num_sms);
-  if (ws_bytes < L.total) return LAGP_ERR_INVALID_ARG;
+  const int Qpad = mix_qpad(b.Mmax, 1);
+  const size_t pred = predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms);
+  const int G = mix_fit(mix_batch_grid(b, di.num_sms), ws_bytes, b.pmax, b.nmax, Qpad, b.idx_total, pred, di.num_sms);
+  if (G < 1) return LAGP_ERR_INVALID_ARG;
+  const MixLayout L = mix_layout(G, b.pmax, b.nmax, Qpad, b.idx_total, pred);
   MixParams P;
   P.X = nullptr; P.Z = nullptr; P.N = 0; P.p = b.pmax; P.XX = b.XX; P.T = b.T; P.cand = b.cand;
   P.M = b.Mmax; P.Qpad = Qpad; P.Mpad = 2 * Qpad; P.n0 = 0; P.n = b.nmax;

@@ -102,8 +102,8 @@ Offsets dev_offsets(int64_t T, int32_t nmax) {
   return o;
 }
 
-// Workspace of the worst batch a slot accepts: max_batch locations, all with nmax and Mmax,
-// spread over every design (the largest N and p).
+// Workspace of the worst batch a slot accepts: max_batch locations, all with nmax and Mmax, on
+// designs of the largest N and p.
 size_t worst_workspace(const lagp_design_desc *designs, int nd, int32_t method, int32_t precision,
                        int32_t nmax, int32_t Mmax, int64_t max_batch) {
   std::vector<int32_t> dof(max_batch), n(max_batch, nmax), m(max_batch);
@@ -111,7 +111,16 @@ size_t worst_workspace(const lagp_design_desc *designs, int nd, int32_t method, 
     dof[t] = (int32_t)(t % nd);
     m[t] = (int32_t)std::min<int64_t>(Mmax, designs[dof[t]].N);
   }
-  return lagp_predict_batch_workspace_bytes(designs, nd, max_batch, dof.data(), n.data(), m.data(),
+  const size_t own = lagp_predict_batch_workspace_bytes(designs, nd, max_batch, dof.data(), n.data(),
+                                                        m.data(), method, precision);
+  if (!own) return 0;
+  std::vector<lagp_design_desc> most(designs, designs + nd);  // (the query reads no device memory)
+  int64_t N = 0;
+  int32_t p = 0;
+  for (const auto &d : most) N = std::max(N, d.N), p = std::max(p, d.p);
+  for (auto &d : most) d.N = N, d.p = p;
+  std::fill(m.begin(), m.end(), (int32_t)std::min<int64_t>(Mmax, N));
+  return lagp_predict_batch_workspace_bytes(most.data(), nd, max_batch, dof.data(), n.data(), m.data(),
                                             method, precision);
 }
 
