@@ -541,7 +541,8 @@ struct RescoreCtx {
 // scratch, and each listed candidate's u = L^{-1} k_c is obtained by forward substitution
 // (one warp per candidate), giving v_j(c) = 1 + g - |u|^2 and cov_j(x, c) = k(x, c) - u.u_x.
 // On return (all threads, after a barrier): *bn / *bd is the CTA's best FP64 score as a
-// fraction, *br its global rank (0x7fffffff if none), or *R.fail set (factor not PD).
+// fraction, *br its global rank (0x7fffffff if none), or *R.fail set (factor not PD; FxArith also:
+// more candidates than the list holds).
 template <class A>
 __device__ __noinline__ void rescore_fp64(const RescoreCtx &R, float B1, double *bn_out, double *bd_out,
                              int *br_out) {
@@ -557,6 +558,14 @@ __device__ __noinline__ void rescore_fp64(const RescoreCtx &R, float B1, double 
     if (sc >= B1 * (1.0f - 2.0f * R.delta)) {
       const int pos = atomicAdd(R.nlist, 1);
       if (pos < RESCORE_CAP) R.rlist[pos] = c;
+    }
+  }
+  if constexpr (A::kFixed) {  // more near-ties than the list holds: the recursion's work
+    __syncthreads();
+    if (*R.nlist > RESCORE_CAP) {
+      if (tid == 0) *R.fail = 1;
+      __syncthreads();
+      return;
     }
   }
   // FP64 factor of the current design with k(x) as an extra column (lower triangle)

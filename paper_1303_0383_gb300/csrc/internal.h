@@ -67,9 +67,20 @@ int select_default_grid(int64_t T, int num_sms);
 size_t select_scratch_bytes_for_grid(int G, int32_t p, int32_t n, int32_t ncand);
 int select_launch_on_grid(const SelectArgs &a, void *ws, size_t ws_bytes, int G,
                           cudaStream_t stream);
+// The FP64 recursion on the *count locations (queue positions, both device) in `list`, of a uniform
+// launch (a) or of a batch (b): what the ALC screen left to it.  queue: a zeroed counter.
+struct BatchLaunch;
+struct HandedList {
+  int *queue;
+  const int32_t *list;
+  const int *count;
+};
+int select_listed_launch(const SelectArgs *a, const BatchLaunch *b, const HandedList &h, void *scratch,
+                         size_t bytes, cudaStream_t stream);
 
 // Mixed-precision variant of kernels (b)+(c) (ALC): float-float screen, FP64 decisions.
-size_t select_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms);
+size_t select_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int32_t precision, int num_sms);
+bool select_mixed_fits(const SelectArgs &a, size_t ws_bytes);  // room for one CTA per SM at least
 int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream);
 
 // ALC in the paper's own form (explicit K_j^{-1}, partition inverse updates), FP64:
@@ -160,6 +171,7 @@ int select_mspe_mixed_prepare();
 size_t select_batch_workspace_bytes(const BatchLaunch &b, int num_sms);
 int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream);
 size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b);
+bool select_mixed_batch_fits(const BatchLaunch &b, size_t ws_bytes);
 int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream);
 size_t select_mspe_batch_workspace_bytes(const BatchLaunch &b, int G);
 int select_mspe_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, int G, cudaStream_t stream);

@@ -64,6 +64,8 @@ struct SelParams {
   int nstart;
   double r_min;          // > 1: stopping rule of Sec. 6 (ALC); 0: the design has n points
   int32_t *n_out;        // design sizes (T) when r_min > 1
+  const int32_t *list;   // queue positions to take (*count of them), or nullptr: all T
+  const int *count;
 };
 
 // ALC scores are compared as fractions cov^2 / v without dividing: a/da beats b/db when
@@ -100,12 +102,13 @@ __global__ void __launch_bounds__(SB, 2) select_fp64_kernel(SelParams P) {
                 dynamic_smem_bytes() + 1u, 25))
     return;
 
+  const int64_t T = P.list ? *P.count : P.T;
   for (;;) {
     __syncthreads();
     if (tid == 0) sh_loc = atomicAdd(P.queue, 1);
     __syncthreads();
-    if (sh_loc >= P.T) break;
-    const LocParams L = resolve_loc(P.B, sh_loc, P.X, P.Z, P.XX, P.p, P.n, P.M, P.n0, P.theta,
+    if (sh_loc >= T) break;
+    const LocParams L = resolve_loc(P.B, P.list ? P.list[sh_loc] : sh_loc, P.X, P.Z, P.XX, P.p, P.n, P.M, P.n0, P.theta,
                                     P.g, P.cand, P.idx, P.N);
     const int64_t loc = L.loc;
     const int n = L.n, p = L.p, M = L.M;
@@ -263,10 +266,7 @@ __global__ void __launch_bounds__(SB, 2) select_fp64_kernel(SelParams P) {
   }
 }
 
-int sel_grid(int64_t T, int num_sms) {
-  int64_t g = (int64_t)num_sms * 2;
-  return (int)(T < g ? (T > 0 ? T : 1) : g);
-}
+int sel_grid(int64_t T, int num_sms) { return (int)rec_grid(T, num_sms); }
 
 int mpad_of(int M) { return (int)align_up((size_t)M, 32); }
 
@@ -286,14 +286,15 @@ size_t select_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, in
                                    : select_mspe_workspace_bytes(T, p, n, ncand, num_sms);
   const size_t own = select_scratch_bytes_for_grid(sel_grid(T, num_sms), p, n, ncand);
   if (method == LAGP_NN) return std::max(own, predict_fp64_workspace_bytes(T, n, num_sms));
-  const size_t scr = select_mixed_workspace_bytes(T, p, n, ncand, num_sms);
+  const size_t scr = select_mixed_workspace_bytes(T, p, n, ncand, precision, num_sms);
   return precision == LAGP_MIXED || scr > own ? scr : own;
 }
 
 // FP64 ALC designs by the fixed-point screen (select_mixed.cu), which resolves v_j(c) >= g at
 // least as finely as FP64 does as long as g is well above its unit (2^-57 of 1 + g) and decides
 // near ties in this file's own arithmetic; smaller nuggets, where a candidate's v may be
-// rounding noise, the stopping rule, NN and callers with the smaller workspace stay here.
+// rounding noise, the stopping rule, NN and callers with the smaller workspace stay here, and so
+// does every location that the screen lists (select_listed_launch).
 // GB300: 4001 2-d locations, n = 50 of 1000, whole call: 23.1 -> 5.95 ms.
 static bool screened(int32_t method, double g, double r_min) {
   return method == LAGP_ALC && g >= 9.3132257461547852e-10 && r_min == 0.0;  // 2^-30
@@ -323,8 +324,7 @@ int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t s
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  if (screened(a.method, a.g, a.r_min) &&
-      ws_bytes >= select_mixed_workspace_bytes(a.T, a.p, a.n, a.M, di.num_sms))
+  if (screened(a.method, a.g, a.r_min) && select_mixed_fits(a, ws_bytes))
     return select_mixed_launch(a, ws, ws_bytes, stream);
   if (a.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(a.T, a.n, di.num_sms)) {
     PredictArgs pa = nn_args(a.XX, a.T, a.n, a.cand, a.M, a.mean, a.s2, a.var, a.idx, a.status);
@@ -339,9 +339,46 @@ int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t s
 int select_default_grid(int64_t T, int num_sms) { return sel_grid(T, num_sms); }
 
 size_t select_scratch_bytes_for_grid(int G, int32_t p, int32_t n, int32_t ncand) {
-  const size_t Mpad = (size_t)mpad_of(ncand);
-  return 256 + align_up((size_t)G * (size_t)n * Mpad * sizeof(double), 256) +
-         align_up((size_t)G * (size_t)p * Mpad * sizeof(double), 256);
+  return 256 + rec_slots_bytes(G, p, n, ncand);
+}
+
+// The arguments of a uniform launch, and of a batch.
+static SelParams sel_params(const SelectArgs &a) {
+  SelParams P = {};
+  P.X = a.X; P.Z = a.Z; P.N = a.N; P.p = a.p; P.XX = a.XX; P.T = a.T; P.cand = a.cand;
+  P.M = a.M; P.Mpad = mpad_of(a.M); P.n0 = a.n0; P.n = a.n; P.method = a.method;
+  P.theta = a.theta;
+  P.g = a.g;
+  P.nmax = a.n;
+  P.pmax = a.p;
+  P.B = BatchView{nullptr, nullptr, nullptr, 0, a.theta_loc, nullptr};
+  P.start = a.start; P.nstart = a.nstart;
+  P.r_min = a.r_min; P.n_out = a.n_out;
+  P.mean = a.mean; P.s2 = a.s2; P.var = a.var; P.idx = a.idx; P.status = a.status;
+  return P;
+}
+static SelParams sel_params(const BatchLaunch &b) {
+  SelParams P = {};
+  P.p = b.pmax; P.XX = b.XX; P.T = b.T; P.cand = b.cand;
+  P.M = b.Mmax; P.Mpad = mpad_of(b.Mmax); P.n = b.nmax; P.method = b.method;
+  P.theta = 1.0; P.nmax = b.nmax; P.pmax = b.pmax;
+  P.B = BatchView{b.designs, b.locs, b.order, b.ldxx, nullptr, nullptr};
+  P.mean = b.mean; P.s2 = b.s2; P.var = b.var; P.idx = b.idx; P.status = b.status;
+  return P;
+}
+
+// The recursion on G CTAs; slots: rec_slots_bytes(G) of scratch, P.queue a zeroed counter.
+static int sel_run(SelParams P, int G, void *slots, const DevInfo &di, cudaStream_t stream) {
+  P.U = static_cast<double *>(slots);
+  P.Xc = reinterpret_cast<double *>(static_cast<char *>(slots) +
+                                    align_up((size_t)G * P.nmax * P.Mpad * sizeof(double), 256));
+  const size_t smem = sel_smem_bytes(P.Mpad, P.nmax);
+  if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
+  const int st = allow_smem(reinterpret_cast<const void *>(select_fp64_kernel), di);
+  if (st) return st;
+  select_fp64_kernel<<<G, SB, smem, stream>>>(P);
+  g_launches.fetch_add(1);
+  return cuda_status(cudaGetLastError());
 }
 
 int select_launch_on_grid(const SelectArgs &a, void *ws, size_t ws_bytes, int G,
@@ -354,32 +391,25 @@ int select_launch_on_grid(const SelectArgs &a, void *ws, size_t ws_bytes, int G,
   st = exp_table_upload();
   if (st) return st;
   if (ws_bytes < select_scratch_bytes_for_grid(G, a.p, a.n, a.M)) return LAGP_ERR_INVALID_ARG;
-  const int Mpad = mpad_of(a.M);
-  char *w = static_cast<char *>(ws);
-  SelParams P;
-  P.X = a.X; P.Z = a.Z; P.N = a.N; P.p = a.p; P.XX = a.XX; P.T = a.T; P.cand = a.cand;
-  P.M = a.M; P.Mpad = Mpad; P.n0 = a.n0; P.n = a.n; P.method = a.method;
-  P.theta = a.theta;
-  P.g = a.g;
-  P.nmax = a.n;
-  P.pmax = a.p;
-  P.B = BatchView{nullptr, nullptr, nullptr, 0, a.theta_loc, nullptr};
-  P.start = a.start; P.nstart = a.nstart;
-  P.r_min = a.r_min; P.n_out = a.n_out;
-  P.mean = a.mean; P.s2 = a.s2; P.var = a.var; P.idx = a.idx; P.status = a.status;
-  P.queue = reinterpret_cast<int *>(w);
-  P.U = reinterpret_cast<double *>(w + 256);
-  P.Xc = reinterpret_cast<double *>(w + 256 + align_up((size_t)G * a.n * Mpad * sizeof(double), 256));
-  const size_t smem = sel_smem_bytes(Mpad, a.n);
-  if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  st = allow_smem(reinterpret_cast<const void *>(select_fp64_kernel), di);
-  if (st) return st;
-  cudaError_t e;
-  e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);   // the work counter starts at zero
+  SelParams P = sel_params(a);
+  P.queue = static_cast<int *>(ws);
+  const cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);   // the work counter starts at zero
   if (e != cudaSuccess) return cuda_status(e);
-  select_fp64_kernel<<<G, SB, smem, stream>>>(P);
-  g_launches.fetch_add(1);
-  return cuda_status(cudaGetLastError());
+  return sel_run(P, G, static_cast<char *>(ws) + 256, di, stream);
+}
+
+int select_listed_launch(const SelectArgs *a, const BatchLaunch *b, const HandedList &h, void *scratch,
+                         size_t bytes, cudaStream_t stream) {
+  DevInfo di;
+  int st = dev_info(&di);
+  if (st) return st;
+  st = exp_table_upload();
+  if (st) return st;
+  SelParams P = a ? sel_params(*a) : sel_params(*b);
+  const int64_t G = rec_fit(P.T, bytes, P.pmax, P.nmax, P.M, di.num_sms);
+  if (G < 1) return LAGP_ERR_INVALID_ARG;
+  P.queue = h.queue; P.list = h.list; P.count = h.count;
+  return sel_run(P, (int)G, scratch, di, stream);
 }
 
 int select_max_ctas(int32_t method, int32_t precision) {
@@ -418,7 +448,7 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
     return b.precision == LAGP_MIXED ? select_mspe_mixed_batch_launch(b, ws, ws_bytes, G, stream)
                                      : select_mspe_batch_launch(b, ws, ws_bytes, G, stream);
   if ((b.precision == LAGP_MIXED && b.method == LAGP_ALC) ||
-      (screened(b.method, b.gmin, 0.0) && ws_bytes >= select_mixed_batch_workspace_bytes(b)))
+      (screened(b.method, b.gmin, 0.0) && select_mixed_batch_fits(b, ws_bytes)))
     return select_mixed_batch_launch(b, ws, ws_bytes, stream);
   if (b.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms)) {
     PredictArgs pa = nn_args(b.XX, b.T, b.nmax, b.cand, b.Mmax, b.mean, b.s2, b.var, b.idx, b.status);
@@ -427,29 +457,11 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
     return predict_fp64_launch(pa, ws, ws_bytes, stream);
   }
   if (ws_bytes < select_scratch_bytes_for_grid(G, b.pmax, b.nmax, b.Mmax)) return LAGP_ERR_INVALID_ARG;
-  const int Mpad = mpad_of(b.Mmax);
-  char *w = static_cast<char *>(ws);
-  SelParams P;
-  P.X = nullptr; P.Z = nullptr; P.N = 0; P.p = b.pmax; P.XX = b.XX; P.T = b.T; P.cand = b.cand;
-  P.M = b.Mmax; P.Mpad = Mpad; P.n0 = 0; P.n = b.nmax; P.method = b.method;
-  P.theta = 1.0; P.g = 0.0; P.nmax = b.nmax; P.pmax = b.pmax;
-  P.B = BatchView{b.designs, b.locs, b.order, b.ldxx, nullptr, nullptr};
-  P.start = nullptr; P.nstart = 0;
-  P.r_min = 0.0; P.n_out = nullptr;
-  P.mean = b.mean; P.s2 = b.s2; P.var = b.var; P.idx = b.idx; P.status = b.status;
-  P.queue = reinterpret_cast<int *>(w);
-  P.U = reinterpret_cast<double *>(w + 256);
-  P.Xc = reinterpret_cast<double *>(w + 256 + align_up((size_t)G * b.nmax * Mpad * sizeof(double), 256));
-  const size_t smem = sel_smem_bytes(Mpad, b.nmax);
-  if (smem > di.smem_optin) return LAGP_ERR_INVALID_ARG;
-  st = allow_smem(reinterpret_cast<const void *>(select_fp64_kernel), di);
-  if (st) return st;
-  cudaError_t e;
-  e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
+  SelParams P = sel_params(b);
+  P.queue = static_cast<int *>(ws);
+  const cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_status(e);
-  select_fp64_kernel<<<G, SB, smem, stream>>>(P);
-  g_launches.fetch_add(1);
-  return cuda_status(cudaGetLastError());
+  return sel_run(P, G, static_cast<char *>(ws) + 256, di, stream);
 }
 
 int select_prepare() {

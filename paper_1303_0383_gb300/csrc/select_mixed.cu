@@ -17,7 +17,8 @@
 // Otherwise the screen's best is taken.  DELTA = 1e-5 is about five times the largest
 // discrepancy between the FP64 scores and those of a screen of 46 bits, by emulation (2e-6
 // of the best score); with the fixed-point screen the factor and the re-score round exactly as
-// the FP64 recursion does, so that every decision is that recursion's.
+// the FP64 recursion does, so that every decision is that recursion's.  A location that the fixed
+// point does not resolve as FP64 does is listed, and the recursion itself takes it afterwards.
 //
 // Each thread screens a pair of candidates, and a step needs one block barrier: every thread
 // merges the per-warp best/second-best results and derives the step's pivot scalars itself.
@@ -64,6 +65,8 @@ struct MixParams {
   int smem;      // bytes of dynamic shared memory
   void *Xr;      // slots of p x Qpad pairs: candidate coordinates minus x
   double *A;     // slots of n x (n + 2): FP64 factorisation
+  int32_t *list; // FxArith: queue positions left to the FP64 recursion, *nlist of them
+  int *nlist;
   int *queue;
   int *rescores; // count of FP64 re-score passes (diagnostics)
   const int32_t *start;  // saved start designs (T x nstart design indices), or nullptr
@@ -79,9 +82,10 @@ struct MixParams {
 
 // FxArith: a location's state (one CTA): v = 1+g, cov_0(x, c) = K(x, c) in FP64, the coordinates
 // relative to x, in formats set by the largest coordinate difference and K(x, c) (compared by
-// the high words of their doubles, which are ordered like the values).  Returns whether every
-// step is to be decided in FP64: coordinates that are not finite, or spread so far that the
-// format's resolution, 2^(b-58), falls short of FP64's.
+// the high words of their doubles, which are ordered like the values).  Returns whether the
+// location is the FP64 recursion's: coordinates that are not finite, or spread so far that the
+// format's resolution, 2^(b-58), falls short of FP64's (beyond b = 14 distances lose whole bits, and
+// the correlations are no covariance any more).
 template <int MBT>
 __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, const double *etab, int4 *vp,
                                          int4 *cp, int4 *Xr, unsigned char *used, int Qpad, FxFormat &F) {
@@ -289,9 +293,10 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
     if (tid < p) xl[tid] = L.x[tid];
     if (tid == 0) sh_fail = 0;
     __syncthreads();
-    bool exact = false;  // (FxArith) every step is decided in FP64
+    bool hand = false;  // (FxArith) the location is left to the FP64 recursion
     if constexpr (A::kFixed) {
-      exact = fx_location<MBT>(L, xl, etab, vp, cp, Xr, used, Qpad, fx);
+      hand = fx_location<MBT>(L, xl, etab, vp, cp, Xr, used, Qpad, fx);
+      if (hand && tid == 0) sh_fail = 1;
     } else {
       // coordinates relative to x over sqrt(theta), v = 1+g, cov_0(x,c) = K(x,c) in FP64, all as
       // float-float pairs
@@ -345,7 +350,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
     // the pivot record in use, and whether it holds the step's pivot already
     int active = 0;
     bool have = false;
-    for (int j = 0; j < n; j++) {
+    for (int j = hand ? n : 0; j < n; j++) {
       const int s = (j < n0e) ? (P.start ? dr[j] : j) : best;
       if (s < 0) {  // nothing admissible left (the same for every thread)
         if (tid == 0) sh_fail = 1;
@@ -488,10 +493,9 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       float delta = DELTA;
       if constexpr (A::kFixed) {
         if (K1) delta += scalbnf(1.0f, 13 - csum) / fmaxf(fabsf(fx_to_float(A::get64(cp, best))), 1.0f);
-        if (exact) delta = 1.0f;
       }
       const float B1 = __uint_as_float(K1 - 1u), B2 = __uint_as_float(K2 - 1u);
-      const bool near = K1 && ((K2 && B2 >= B1 * (1.0f - delta)) || exact);
+      const bool near = K1 && K2 && B2 >= B1 * (1.0f - delta);
       if (!near) continue;
       // ---- FP64 re-score of the near-tied candidates (rare) ----
       if (tid == 0 && crank == 0 && P.rescores) atomicAdd(P.rescores, 1);
@@ -532,7 +536,10 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
     if constexpr (CLU) cg::this_cluster().sync();
     else __syncthreads();
     // the design (design indices), or -1 when a step failed; kernel (c) (predict.cu)
-    // evaluates the predictive equations on it in FP64
+    // evaluates the predictive equations on it in FP64.  (FxArith: whatever stopped the screen, the
+    // recursion decides whether the location fails.)
+    if constexpr (A::kFixed)
+      if (sh_fail && tid == 0) P.list[atomicAdd(P.nlist, 1)] = qloc;
     if (crank == 0) {
       for (int i = tid; i < n; i += MBT)
         L.idx[i] = (sh_fail || i >= ne || !LAGP_CHK(dr[i], M, 16)) ? -1 : L.cand[dr[i]];
@@ -678,12 +685,15 @@ int mix_cluster_grid(int64_t T, MixVariant v, size_t smem, const DevInfo &di, in
   return LAGP_OK;
 }
 
-// The screen, then kernel (c) on the designs it selected.
-int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, int32_t *user_idx,
-            const DevInfo &di, cudaStream_t stream) {
+// The screen, then kernel (c) on the designs it selected, then (FP64) the recursion on the listed
+// locations, whose designs are -1 until then.
+int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, size_t ws_bytes, int32_t *user_idx,
+            const SelectArgs *sa, const BatchLaunch *sb, const DevInfo &di, cudaStream_t stream) {
   P.queue = reinterpret_cast<int *>(w);
+  P.nlist = reinterpret_cast<int *>(w + 64);
   P.rescores = reinterpret_cast<int *>(w + 256);
-  char *o = w + 512;
+  P.list = reinterpret_cast<int32_t *>(w + 512);
+  char *o = w + 512 + L.list;
   P.U = o;
   o += L.u;
   P.Xr = o;
@@ -711,7 +721,7 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, int32
     if (e != cudaSuccess) return cuda_status(e);
     if (k * tmem_cols(v.MBT) > 512) return LAGP_ERR_CUDA;
   }
-  e = cudaMemsetAsync(w, 0, 512, stream);  // work counter and re-score counter
+  e = cudaMemsetAsync(w, 0, 512, stream);  // the counters
   if (e != cudaSuccess) return cuda_status(e);
   cudaLaunchAttribute attr[1];
   const cudaLaunchConfig_t cfg = mix_config(v, G, smem, stream, attr);
@@ -727,7 +737,11 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, int32
   pa.B.n_loc = P.n_out;  // adaptive designs: kernel (c) on each location's own size
   pa.recip = v.fixed;    // FP64: the recursion's own rounding, and no design where it fails
   pa.mean = P.mean; pa.s2 = P.s2; pa.var = P.var; pa.status = P.status;
-  return predict_fp64_launch(pa, o, L.pred, stream);
+  const int sp = predict_fp64_launch(pa, o, L.pred, stream);
+  if (sp || !v.fixed) return sp;
+  const size_t used = 512 + L.list;
+  return select_listed_launch(sa, sb, HandedList{reinterpret_cast<int *>(w + 128), P.list, P.nlist}, w + used,
+                              ws_bytes - used, stream);
 }
 
 // A batch's instance suits its largest candidate count; the grid is the batch's share of
@@ -744,8 +758,21 @@ int mix_batch_grid(const BatchLaunch &b, int num_sms) {
 
 int select_mixed_check_take(CheckRec *out) { return check_take_here(out); }
 
-size_t select_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms) {
-  return mix_asked_bytes(T, p, n, ncand, T * n, predict_fp64_workspace_bytes(T, n, num_sms), num_sms, true);
+size_t select_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int32_t precision, int num_sms) {
+  const bool fixed = precision == LAGP_FP64;
+  return mix_asked_bytes(T, p, n, ncand, T * n, predict_fp64_workspace_bytes(T, n, num_sms), num_sms, !fixed,
+                         fixed ? T : 0);
+}
+
+// The grid of a uniform launch (not the cluster form) in ws_bytes, 0: no room.
+static int mix_uniform_fit(const SelectArgs &a, MixVariant v, size_t ws_bytes, const DevInfo &di) {
+  return mix_fit(mix_grid(a.T, di.num_sms, v), ws_bytes, a.p, a.n, mix_qpad(a.M, 1), a.T * a.n,
+                 predict_fp64_workspace_bytes(a.T, a.n, di.num_sms), di.num_sms, v.fixed ? a.T : 0);
+}
+
+bool select_mixed_fits(const SelectArgs &a, size_t ws_bytes) {
+  DevInfo di;
+  return dev_info(&di) == LAGP_OK && mix_uniform_fit(a, mix_variant(a.M, 1, a.precision == LAGP_FP64), ws_bytes, di) > 0;
 }
 
 int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -766,9 +793,9 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
     if (st) return st;
   }
   const size_t pred = predict_fp64_workspace_bytes(a.T, a.n, di.num_sms);
-  if (v.CL == 1) G = mix_fit(G, ws_bytes, a.p, a.n, Qpad, a.T * a.n, pred, di.num_sms);
+  if (v.CL == 1) G = mix_uniform_fit(a, v, ws_bytes, di);
   if (G < 1) return LAGP_ERR_INVALID_ARG;
-  const MixLayout L = mix_layout(G, a.p, a.n, Qpad, a.T * a.n, pred);
+  const MixLayout L = mix_layout(G, a.p, a.n, Qpad, a.T * a.n, pred, v.fixed ? a.T : 0);
   if (ws_bytes < L.total) return LAGP_ERR_INVALID_ARG;
   MixParams P;
   P.X = a.X; P.Z = a.Z; P.N = a.N; P.p = a.p; P.XX = a.XX; P.T = a.T; P.cand = a.cand;
@@ -779,14 +806,26 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
   P.start = a.start; P.nstart = a.nstart;
   P.r_min = a.r_min; P.n_out = a.n_out;
   P.mean = a.mean; P.s2 = a.s2; P.var = a.var; P.status = a.status;
-  return mix_run(P, v, L, G, static_cast<char *>(ws), a.idx, di, stream);
+  return mix_run(P, v, L, G, static_cast<char *>(ws), ws_bytes, a.idx, &a, nullptr, di, stream);
 }
 
 size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b) {
   DevInfo di;
   const int sms = dev_info(&di) == LAGP_OK ? di.num_sms : 152;
   return mix_asked_bytes(b.T, b.pmax, b.nmax, b.Mmax, b.idx_total, predict_fp64_workspace_bytes(b.T, b.nmax, sms), sms,
-                         false);
+                         false, b.precision == LAGP_FP64 ? b.T : 0);
+}
+
+// A batch's grid in ws_bytes, 0: no room.
+static int mix_batch_fit(const BatchLaunch &b, size_t ws_bytes, const DevInfo &di) {
+  return mix_fit(mix_batch_grid(b, di.num_sms), ws_bytes, b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.idx_total,
+                 predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms), di.num_sms,
+                 b.precision == LAGP_FP64 ? b.T : 0);
+}
+
+bool select_mixed_batch_fits(const BatchLaunch &b, size_t ws_bytes) {
+  DevInfo di;
+  return dev_info(&di) == LAGP_OK && mix_batch_fit(b, ws_bytes, di) > 0;
 }
 
 // (Locations grouped by candidate count, one launch of a fitting instance each, measured slower:
@@ -797,11 +836,11 @@ int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, c
   if (st) return st;
   st = exp_table_upload();  // this translation unit's copy of the exp constants
   if (st) return st;
-  const int Qpad = mix_qpad(b.Mmax, 1);
-  const size_t pred = predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms);
-  const int G = mix_fit(mix_batch_grid(b, di.num_sms), ws_bytes, b.pmax, b.nmax, Qpad, b.idx_total, pred, di.num_sms);
+  const int Qpad = mix_qpad(b.Mmax, 1), G = mix_batch_fit(b, ws_bytes, di);
   if (G < 1) return LAGP_ERR_INVALID_ARG;
-  const MixLayout L = mix_layout(G, b.pmax, b.nmax, Qpad, b.idx_total, pred);
+  const MixLayout L = mix_layout(G, b.pmax, b.nmax, Qpad, b.idx_total,
+                                 predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms),
+                                 b.precision == LAGP_FP64 ? b.T : 0);
   MixParams P;
   P.X = nullptr; P.Z = nullptr; P.N = 0; P.p = b.pmax; P.XX = b.XX; P.T = b.T; P.cand = b.cand;
   P.M = b.Mmax; P.Qpad = Qpad; P.Mpad = 2 * Qpad; P.n0 = 0; P.n = b.nmax;
@@ -811,7 +850,7 @@ int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, c
   P.start = nullptr; P.nstart = 0;
   P.r_min = 0.0; P.n_out = nullptr;
   P.mean = b.mean; P.s2 = b.s2; P.var = b.var; P.status = b.status;
-  return mix_run(P, mix_batch_variant(b), L, G, static_cast<char *>(ws), b.idx, di, stream);
+  return mix_run(P, mix_batch_variant(b), L, G, static_cast<char *>(ws), ws_bytes, b.idx, nullptr, &b, di, stream);
 }
 
 int select_mixed_prepare() {

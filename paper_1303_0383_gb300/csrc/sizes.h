@@ -34,48 +34,67 @@ constexpr int kMixTop[2] = {512, 1024};
 inline int mix_threads(int M) { return M <= kMixTop[0] ? 128 : M <= kMixTop[1] ? 256 : 512; }
 
 struct MixLayout {
-  size_t u, xr, a, idx, pred, total;
+  size_t list, u, xr, a, idx, pred, total;
 };
 
-// [queue | re-score counter | U | Xr | A | design indices | kernel (c) workspace] of G CTAs, each
+// [counters, 512 bytes | list | U | Xr | A | design indices | kernel (c) workspace] of G CTAs, each
 // with a slot of n x Qpad factor rows and p x Qpad coordinates (16 bytes per pair) and of the
-// n x (n + 2) FP64 factorisation; pred: kernel (c)'s bytes.
-inline MixLayout mix_layout(int64_t G, int p, int n, int Qpad, int64_t idx_total, size_t pred) {
+// n x (n + 2) FP64 factorisation; pred: kernel (c)'s bytes.  listed: the locations that the list
+// of those left to the FP64 recursion has room for (FP64: all of them; mixed: 0).  The recursion
+// runs last, in all that follows the list.
+inline MixLayout mix_layout(int64_t G, int p, int n, int Qpad, int64_t idx_total, size_t pred, int64_t listed) {
   MixLayout L;
+  L.list = align_up((size_t)listed * sizeof(int32_t), 256);
   L.u = align_up((size_t)G * n * Qpad * 16, 256);
   L.xr = align_up((size_t)G * p * Qpad * 16, 256);
   L.a = align_up((size_t)G * n * (n + 2) * sizeof(double), 256);
   L.idx = align_up((size_t)idx_total * sizeof(int32_t), 256);
   L.pred = pred;
-  L.total = 256 + 256 + L.u + L.xr + L.a + L.idx + L.pred;
+  L.total = 512 + L.list + L.u + L.xr + L.a + L.idx + L.pred;
   return L;
+}
+
+// Scratch of the FP64 recursion's slots (select.cu): n x Mpad factor rows and p x Mpad coordinates.
+inline size_t rec_slots_bytes(int64_t G, int p, int n, int M) {
+  const size_t Mpad = align_up((size_t)M, 32);
+  return align_up((size_t)G * (size_t)n * Mpad * sizeof(double), 256) +
+         align_up((size_t)G * (size_t)p * Mpad * sizeof(double), 256);
+}
+// CTAs of the recursion for T locations: two per SM.
+inline int64_t rec_grid(int64_t T, int num_sms) { return std::min<int64_t>(2 * (int64_t)num_sms, T > 0 ? T : 1); }
+// Of those, as many as fit in `bytes`.
+inline int64_t rec_fit(int64_t T, size_t bytes, int p, int n, int M, int num_sms) {
+  return std::min<int64_t>(rec_grid(T, num_sms), (int64_t)(bytes / rec_slots_bytes(1, p, n, M)));
 }
 
 // What a workspace query returns: enough for the full grid of every shape that T locations of
 // at most M candidates and n points can take.
 inline size_t mix_asked_bytes(int64_t T, int p, int n, int M, int64_t idx_total, size_t pred, int num_sms,
-                              bool clusters) {
+                              bool clusters, int64_t listed) {
   const int64_t T1 = T > 0 ? T : 1;
   size_t most = 0;
   for (int k = 0; k < 3; k++) {
     const int Mk = k < 2 ? std::min(M, kMixTop[k]) : M;
     const int64_t G = std::min<int64_t>((int64_t)num_sms * (kScrThreads / mix_threads(Mk)), T1);
-    most = std::max(most, mix_layout(G, p, n, mix_qpad(Mk, 1), idx_total, pred).total);
+    most = std::max(most, mix_layout(G, p, n, mix_qpad(Mk, 1), idx_total, pred, listed).total);
   }
   for (int CL = 2; clusters && CL <= kMaxCL; CL *= 2) {
     const int64_t G = std::min<int64_t>((int64_t)num_sms * (kScrThreads / 256), CL * T1);
-    most = std::max(most, mix_layout(G, p, n, mix_qpad(M, CL), idx_total, pred).total);
+    most = std::max(most, mix_layout(G, p, n, mix_qpad(M, CL), idx_total, pred, listed).total);
   }
+  if (listed)
+    most = std::max(most, 512 + mix_layout(0, p, n, 0, 0, 0, listed).list + rec_slots_bytes(rec_grid(T, num_sms), p, n, M));
   return most;
 }
 
 // The largest grid of at most G CTAs that fits in `bytes`; 0 where not even one CTA per SM (or
 // G, if that is fewer) does.
-inline int mix_fit(int64_t G, size_t bytes, int p, int n, int Qpad, int64_t idx_total, size_t pred, int num_sms) {
+inline int mix_fit(int64_t G, size_t bytes, int p, int n, int Qpad, int64_t idx_total, size_t pred, int num_sms,
+                   int64_t listed) {
   const int64_t least = std::min<int64_t>(G, num_sms);
-  if (mix_layout(least, p, n, Qpad, idx_total, pred).total > bytes) return 0;
-  while (mix_layout(G, p, n, Qpad, idx_total, pred).total > bytes) {
-    const MixLayout L = mix_layout(G, p, n, Qpad, idx_total, pred);
+  if (mix_layout(least, p, n, Qpad, idx_total, pred, listed).total > bytes) return 0;
+  while (mix_layout(G, p, n, Qpad, idx_total, pred, listed).total > bytes) {
+    const MixLayout L = mix_layout(G, p, n, Qpad, idx_total, pred, listed);
     const size_t slot = (L.u + L.xr + L.a) / (size_t)G;  // at most 768 / G above a slot's own bytes
     const int64_t over = (int64_t)((L.total - bytes) / (slot + 1)) + 1;
     G = std::max(least, G - over);

@@ -29,23 +29,23 @@ int main() {
         size_t prev = 0;
         for (int M : Ms) {
           if (M < n) continue;
-          const size_t a = mix_asked_bytes(T, 8, n, M, T * n, 256, sms, c);
+          const size_t a = mix_asked_bytes(T, 8, n, M, T * n, 256, sms, c, 0);
           if (a < prev) return bad("mix M", T, n, M);
           prev = a;
           // the grid of the shape that runs, whole, in what was asked for at this or any larger size
           const int64_t G = std::min<int64_t>((int64_t)sms * (kScrThreads / mix_threads(M)), T);
-          if (mix_fit(G, a, 8, n, mix_qpad(M, 1), T * n, 256, sms) != G) return bad("mix fit", T, n, M);
-          if (mix_asked_bytes(T + 1, 8, n, M, (T + 1) * n, 256, sms, c) < a) return bad("mix T", T, n, M);
-          if (n < 256 && M > n && mix_asked_bytes(T, 8, n + 1, M, T * (n + 1), 256, sms, c) < a) return bad("mix n", T, n, M);
+          if (mix_fit(G, a, 8, n, mix_qpad(M, 1), T * n, 256, sms, 0) != G) return bad("mix fit", T, n, M);
+          if (mix_asked_bytes(T + 1, 8, n, M, (T + 1) * n, 256, sms, c, 0) < a) return bad("mix T", T, n, M);
+          if (n < 256 && M > n && mix_asked_bytes(T, 8, n + 1, M, T * (n + 1), 256, sms, c, 0) < a) return bad("mix n", T, n, M);
           // and less of it in less, down to one CTA per SM
           const int64_t least = std::min<int64_t>(G, sms);
-          const size_t small = mix_layout(least, 8, n, mix_qpad(M, 1), T * n, 256).total;
-          if (mix_fit(G, small, 8, n, mix_qpad(M, 1), T * n, 256, sms) != least) return bad("mix least", T, n, M);
-          if (mix_fit(G, small - 1, 8, n, mix_qpad(M, 1), T * n, 256, sms)) return bad("mix refused", T, n, M);
+          const size_t small = mix_layout(least, 8, n, mix_qpad(M, 1), T * n, 256, 0).total;
+          if (mix_fit(G, small, 8, n, mix_qpad(M, 1), T * n, 256, sms, 0) != least) return bad("mix least", T, n, M);
+          if (mix_fit(G, small - 1, 8, n, mix_qpad(M, 1), T * n, 256, sms, 0)) return bad("mix refused", T, n, M);
           if (G > least) {
-            const size_t mid = mix_layout(G - 1, 8, n, mix_qpad(M, 1), T * n, 256).total;
-            const int g = mix_fit(G, mid, 8, n, mix_qpad(M, 1), T * n, 256, sms);
-            if (g < G - 3 || mix_layout(g, 8, n, mix_qpad(M, 1), T * n, 256).total > mid) return bad("mix mid", T, n, M);
+            const size_t mid = mix_layout(G - 1, 8, n, mix_qpad(M, 1), T * n, 256, 0).total;
+            const int g = mix_fit(G, mid, 8, n, mix_qpad(M, 1), T * n, 256, sms, 0);
+            if (g < G - 3 || mix_layout(g, 8, n, mix_qpad(M, 1), T * n, 256, 0).total > mid) return bad("mix mid", T, n, M);
           }
         }
       }
