@@ -85,10 +85,14 @@ struct MixParams {
 // the high words of their doubles, which are ordered like the values).  Returns whether the
 // location is the FP64 recursion's: coordinates that are not finite, or spread so far that the
 // format's resolution, 2^(b-58), falls short of FP64's (beyond b = 14 distances lose whole bits, and
-// the correlations are no covariance any more).
+// the correlations are no covariance any more); and, where the design is to grow (greedy), x so far
+// from every candidate that cov^2 leaves FP64's normal range: there the recursion's scores lose bits
+// or tie at 0, and the screen's, scaled by the largest K(x, c) = 2^-w or more, do not.  cov shrinks
+// from 2^-w by 2^-53 at most before it is rounding error, and is compared as cov^2 v' with v' of
+// 2^-30 or more: 2 (w + 53) + 30 < 1022 for w <= 400.
 template <int MBT>
 __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, const double *etab, int4 *vp,
-                                         int4 *cp, int4 *Xr, unsigned char *used, int Qpad, FxFormat &F) {
+                                         int4 *cp, int4 *Xr, unsigned char *used, int Qpad, bool greedy, FxFormat &F) {
   const int tid = threadIdx.x, p = L.p, M = L.M;
   long long *v = reinterpret_cast<long long *>(vp), *cov = reinterpret_cast<long long *>(cp);
   // e even with 1 + g < 2^(e+1)
@@ -157,7 +161,7 @@ __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, c
     F.fmt[0] = min(2 * b, 62);
     F.fmt[1] = e;
   }
-  return b > 8 || F.odd;
+  return b > 8 || F.odd || (greedy && w > 400);
 }
 
 // MBT threads per CTA, one location per CTA, one or two candidate pairs per thread up to 1024
@@ -295,7 +299,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
     __syncthreads();
     bool hand = false;  // (FxArith) the location is left to the FP64 recursion
     if constexpr (A::kFixed) {
-      hand = fx_location<MBT>(L, xl, etab, vp, cp, Xr, used, Qpad, fx);
+      hand = fx_location<MBT>(L, xl, etab, vp, cp, Xr, used, Qpad, n0e < n, fx);
       if (hand && tid == 0) sh_fail = 1;
     } else {
       // coordinates relative to x over sqrt(theta), v = 1+g, cov_0(x,c) = K(x,c) in FP64, all as
