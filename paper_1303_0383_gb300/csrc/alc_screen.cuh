@@ -147,6 +147,7 @@ struct FfArith {
     const float4 a = reinterpret_cast<const float4 *>(rec + kMaxP)[0];
     return Scalars{ff{a.x, a.y}, ff{a.z, a.w}};
   }
+  static __device__ __forceinline__ ff scalars_ux(const int2 *rec) { return scalars_load(rec).ux; }
   static __device__ __forceinline__ void rec_coord(int2 *rec, int k, const Word *row, int c) {
     const ff x = ff2_get(row, c);
     reinterpret_cast<float2 *>(rec)[k] = make_float2(x.h, x.l);
@@ -251,6 +252,7 @@ struct FxArith {
     const int4 a = o[0], b = o[1];
     return Scalars{FxRsqrt{a.x, a.y, a.z}, FxU{b.x, b.y}, a.w};
   }
+  static __device__ __forceinline__ ff scalars_ux(const int2 *) { return ff{0.0f, 0.0f}; }  // (not kept)
   static __device__ __forceinline__ void rec_coord(int2 *rec, int k, const Word *row, int c) {
     const FxU x = get(row, c);
     rec[k] = make_int2(x.h, x.l);

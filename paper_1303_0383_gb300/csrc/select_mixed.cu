@@ -350,7 +350,6 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
     int best = 0;
     int ne = n;       // the design's size (n, or where the stopping rule ends it)
     ff vx = ff_from_double(L.onepg);  // v_j(x), carried by every thread for the stopping rule
-    int csum = 0;     // (FxArith) cov has been shifted right by this much
     // the pivot record in use, and whether it holds the step's pivot already
     int active = 0;
     bool have = false;
@@ -393,12 +392,10 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
         __syncthreads();
       }
       const int2 *rec = recs + active * recw;
-      if constexpr (A::kFixed) {
-        csum += A::scalars_load(rec).csh;
-      } else if (P.r_min > 0.0) {
+      if (!A::kFixed && P.r_min > 0.0) {
         // Sec. 6 stopping rule: stop before a greedy point whose variance reduction ratio
         // v_j(x) / v_{j+1}(x) (psi cancels) is below r_min; every thread decides alike
-        const ff ux = A::scalars_load(rec).ux;
+        const ff ux = A::scalars_ux(rec);
         const ff vxn = ff_sub(vx, ff_mul(ux, ux));
         if (j >= n0e && ff_to_double(vx) / ff_to_double(vxn) < P.r_min) {
           ne = j;
@@ -492,11 +489,12 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
         if (have) active = buf;
       }
       // Candidates closer than DELTA are decided in FP64.  For the FP64 precision the margin
-      // also covers the FP64 recursion's own rounding of cov_j(x, c) where that is small
-      // (2^-46 of the largest K(x, c)).
+      // also covers the FP64 recursion's own rounding of cov_j(x, c) where that is small: 2^13
+      // units, 2^-46 of the largest K(x, c), or where cov has outgrown that and has been shifted
+      // (Scalars::csh), of the largest u_x u_c, which fills the same 2^59 units.
       float delta = DELTA;
       if constexpr (A::kFixed) {
-        if (K1) delta += scalbnf(1.0f, 13 - csum) / fmaxf(fabsf(fx_to_float(A::get64(cp, best))), 1.0f);
+        if (K1) delta += 8192.0f / fmaxf(fabsf(fx_to_float(A::get64(cp, best))), 1.0f);
       }
       const float B1 = __uint_as_float(K1 - 1u), B2 = __uint_as_float(K2 - 1u);
       const bool near = K1 && K2 && B2 >= B1 * (1.0f - delta);
