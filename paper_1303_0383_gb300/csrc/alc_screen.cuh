@@ -102,6 +102,7 @@ __device__ __forceinline__ void tmem_st4(uint32_t ta, Word v) {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 constexpr int kTmemWords = 128;  // words of one thread
+constexpr size_t kTmemBytes = 256 * 1024;  // of an SM
 // columns of a CTA of nt threads
 __host__ __device__ constexpr int tmem_cols(int nt) { return nt * kTmemWords / 128; }
 

@@ -44,6 +44,9 @@ int dev_info(DevInfo *out) {
     e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     if (e != cudaSuccess) return cuda_status(e);
     d.smem_per_sm = (size_t)v;
+    e = cudaDeviceGetAttribute(&v, cudaDevAttrL2CacheSize, dev);
+    if (e != cudaSuccess) return cuda_status(e);
+    d.l2 = (size_t)v;
     cache[dev] = d;
     have[dev] = true;
   }

@@ -25,6 +25,7 @@ struct DevInfo {
   int num_sms;
   size_t smem_optin;
   size_t smem_per_sm;
+  size_t l2;
 };
 int dev_info(DevInfo *out);
 // Lets a kernel's launches use any dynamic shared memory the device allows.  The limit is state

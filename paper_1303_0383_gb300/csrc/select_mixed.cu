@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
   __shared__ int xr_r[CLU ? kMaxCL : 1];
   __shared__ double red_n[NWARP], red_d[NWARP];
   __shared__ int red_rr[NWARP];
-  __shared__ int sh_loc, sh_fail, sh_nlist;
+  __shared__ int sh_loc, sh_fail, sh_nlist, sh_per;
   __shared__ LocParams L;  // the location's parameters: read where they are used
   __shared__ FxFormat fx;                // the location's formats (FxArith)
   __shared__ unsigned sh_top[3], sh_nwr[3];  // by step: best score key of the warps that are done,
@@ -295,7 +295,14 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
                   dynamic_smem_bytes() + 1u, 20))
       continue;
     if (tid < p) xl[tid] = L.x[tid];
-    if (tid == 0) sh_fail = 0;
+    if (tid == 0) {
+      sh_fail = 0;
+      // a last round of up to 64 pairs would leave nearly all threads idle for its row loops' latency:
+      // rounds of like size then (600 8-d locations, n = 100 of 2100: 11.3 -> 10.3 ms; a larger rest is
+      // better on its own)
+      const int full = NP * MBT, q32 = (Qs + 31) & ~31, rest = q32 % full, rounds = (q32 + full - 1) / full;
+      sh_per = MBT == 512 && q32 > full && rest > 0 && rest <= 64 ? ((q32 + rounds - 1) / rounds + 31) & ~31 : full;
+    }
     __syncthreads();
     bool hand = false;  // (FxArith) the location is left to the FP64 recursion
     if constexpr (A::kFixed) {
@@ -415,9 +422,10 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       // multiple of 32 (all within Qpad; those past Qs only update state nobody reads), each
       // round's in two halves of whole warps
       const int Q32 = (Qs + 31) & ~31;
-      for (int q = tid, k = 0; q - tid < Q32; q += NP * MBT, k += NP) {
-        const int left = Q32 - (q - tid), dq = NP == 1 ? MBT : min(MBT, ((left >> 1) + 31) & ~31);
-        if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, q, b1, r1, b2, k, q + dq < Q32 ? dq : 0);
+      const int per = sh_per;  // pairs of a round
+      for (int base = 0, k = 0; base < Q32; base += per, k += NP) {
+        const int left = min(per, Q32 - base), dq = NP == 1 ? MBT : min(MBT, ((left >> 1) + 31) & ~31);
+        if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, base + tid, b1, r1, b2, k, tid + dq < left ? dq : 0);
       }
       // best and second-best screen scores of the warp; the warp writes the record of its own
       // best candidate as the next step's pivot before the barrier, so that the gather of the
@@ -622,9 +630,10 @@ int mix_cluster_size() {
   return e == 1 || e == 2 || e == 4 || e == 8 ? e : 1;
 }
 
-MixVariant mix_variant(int M, int CL, bool fixed) {
+MixVariant mix_variant(int64_t T, int M, int n, int CL, bool fixed, const DevInfo &di) {
   if (CL > 1) return MixVariant{256, 2, CL, false};
-  return MixVariant{mix_threads(M), mix_qpad(M, 1) <= 128 ? 1 : 2, 1, fixed};
+  const int threads = mix_threads(T, M, n, ScreenChip{di.num_sms, di.l2, di.smem_per_sm + kTmemBytes});
+  return MixVariant{threads, mix_qpad(M, 1) <= 128 ? 1 : 2, 1, fixed};
 }
 
 // Records and dynamic shared memory of a launch whose largest location has Qpad pairs and n
@@ -748,11 +757,13 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, size_
 
 // A batch's instance suits its largest candidate count; the grid is the batch's share of
 // select_max_ctas() CTAs per SM, of that instance's residents.
-MixVariant mix_batch_variant(const BatchLaunch &b) { return mix_variant(b.Mmax, 1, b.precision == LAGP_FP64); }
-int mix_batch_grid(const BatchLaunch &b, int num_sms) {
+MixVariant mix_batch_variant(const BatchLaunch &b, const DevInfo &di) {
+  return mix_variant(b.T, b.Mmax, b.nmax, 1, b.precision == LAGP_FP64, di);
+}
+int mix_batch_grid(const BatchLaunch &b, const DevInfo &di) {
   const int most = select_max_ctas(b.method, b.precision);
   const int ctas = b.ctas_per_sm < 1 || b.ctas_per_sm > most ? most : b.ctas_per_sm;
-  const int64_t g = (int64_t)num_sms * mix_minb(mix_batch_variant(b)) * ctas / most;
+  const int64_t g = (int64_t)di.num_sms * mix_minb(mix_batch_variant(b, di)) * ctas / most;
   return (int)(g < 1 ? 1 : g < b.T ? g : b.T);
 }
 
@@ -774,7 +785,8 @@ static int mix_uniform_fit(const SelectArgs &a, MixVariant v, size_t ws_bytes, c
 
 bool select_mixed_fits(const SelectArgs &a, size_t ws_bytes) {
   DevInfo di;
-  return dev_info(&di) == LAGP_OK && mix_uniform_fit(a, mix_variant(a.M, 1, a.precision == LAGP_FP64), ws_bytes, di) > 0;
+  return dev_info(&di) == LAGP_OK && mix_uniform_fit(a, mix_variant(a.T, a.M, a.n, 1, a.precision == LAGP_FP64, di), ws_bytes,
+                                                       di) > 0;
 }
 
 int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -784,7 +796,8 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  const MixVariant v = mix_variant(a.M, a.precision == LAGP_FP64 ? 1 : mix_cluster_size(), a.precision == LAGP_FP64);
+  const bool fixed = a.precision == LAGP_FP64;
+  const MixVariant v = mix_variant(a.T, a.M, a.n, fixed ? 1 : mix_cluster_size(), fixed, di);
   const int Qpad = mix_qpad(a.M, v.CL);
   int G = mix_grid(a.T, di.num_sms, v);
   if (v.CL > 1) {
@@ -820,7 +833,7 @@ size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b) {
 
 // A batch's grid in ws_bytes, 0: no room.
 static int mix_batch_fit(const BatchLaunch &b, size_t ws_bytes, const DevInfo &di) {
-  return mix_fit(mix_batch_grid(b, di.num_sms), ws_bytes, b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.idx_total,
+  return mix_fit(mix_batch_grid(b, di), ws_bytes, b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.idx_total,
                  predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms), di.num_sms,
                  b.precision == LAGP_FP64 ? b.T : 0);
 }
@@ -852,7 +865,7 @@ int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, c
   P.start = nullptr; P.nstart = 0;
   P.r_min = 0.0; P.n_out = nullptr;
   P.mean = b.mean; P.s2 = b.s2; P.var = b.var; P.status = b.status;
-  return mix_run(P, mix_batch_variant(b), L, G, static_cast<char *>(ws), ws_bytes, b.idx, nullptr, &b, di, stream);
+  return mix_run(P, mix_batch_variant(b, di), L, G, static_cast<char *>(ws), ws_bytes, b.idx, nullptr, &b, di, stream);
 }
 
 int select_mixed_prepare() {

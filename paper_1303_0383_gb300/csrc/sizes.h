@@ -28,10 +28,32 @@ constexpr int kMaxCL = 8;         // CTAs per cluster in the cluster form
 // shared-memory rows after the Mpad = 2 Qpad flag bytes start 16-byte aligned).
 inline int mix_qpad(int M, int CL) { return (int)align_up((size_t)ceil_div(ceil_div(M, 2), CL), 32); }
 
-// Threads per CTA for M candidates: one candidate pair per thread where 256, 512 or 1024 threads
-// cover them.  kMixTop: the largest M of CTAs of 128 and 256 threads.
-constexpr int kMixTop[2] = {512, 1024};
-inline int mix_threads(int M) { return M <= kMixTop[0] ? 128 : M <= kMixTop[1] ? 256 : 512; }
+struct ScreenChip {
+  int num_sms;
+  size_t l2, on_chip;  // bytes of L2, and of shared and tensor memory per SM
+};
+
+// Threads per CTA for T locations of M candidates and n points: one or two candidate pairs per
+// thread, 512 threads per SM in all.  Small CTAs leave fewer threads idle and hide each other's
+// barriers; large ones have a location to themselves sooner and keep fewer factor rows live.  So
+// CTAs of 128 and 256 threads are taken for up to 512 and 1024 candidates, and for half as many again
+// where more than two locations per SM are asked for and the rows of those in flight stay within L2
+// and the chip; with two per SM or fewer, 256 threads from 257 candidates on.  GB300, mixed, 2000 2-d
+// locations, n = 50, in ms for 128 / 256 / 512 threads: M = 400 1.50 / 1.79 / 2.51, 600 2.21 / 2.26 /
+// 3.17, 700 2.25 / 2.53 / 3.22, 1024 3.04 / 2.73 / 3.44, 1100 4.36 / 3.64 / 4.19, 1300 5.07 / 4.06 / 4.39,
+// 1500 5.72 / 4.72 / 4.42; 300 locations, M = 400 0.44 / 0.40 / 0.44; one, 0.27 / 0.24 / 0.24, M = 1100
+// 0.63 / 0.46 / 0.36; 600 8-d ones, n = 100: M = 300 1.67 / 2.08 / 2.48, 500 2.86 / 2.13 / 2.72, 1030 6.54 /
+// 5.67 / 4.23 (rows beyond L2).  kMixTop: the largest M of the first two.
+constexpr int kMixTop[2] = {768, 1344};
+inline int mix_threads(int64_t T, int M, int n, const ScreenChip &c) {
+  const int Qpad = mix_qpad(M, 1);
+  const bool many = T > 2 * (int64_t)c.num_sms;
+  const double room = (double)c.l2 + (double)c.num_sms * c.on_chip;
+  auto fits = [&](int k) { return 16.0 * k * c.num_sms * n * Qpad <= room; };  // k locations per SM
+  if (Qpad <= 128 || (many && 2 * Qpad <= kMixTop[0] && fits(4))) return 128;
+  if (2 * Qpad <= 1024 || (many && 2 * Qpad <= kMixTop[1] && fits(2))) return 256;
+  return 512;
+}
 
 struct MixLayout {
   size_t list, u, xr, a, idx, pred, total;
@@ -67,15 +89,15 @@ inline int64_t rec_fit(int64_t T, size_t bytes, int p, int n, int M, int num_sms
   return std::min<int64_t>(rec_grid(T, num_sms), (int64_t)(bytes / rec_slots_bytes(1, p, n, M)));
 }
 
-// What a workspace query returns: enough for the full grid of every shape that T locations of
-// at most M candidates and n points can take.
+// What a workspace query returns: enough for the full grid of every shape, for T locations of at
+// most M candidates and n points.
 inline size_t mix_asked_bytes(int64_t T, int p, int n, int M, int64_t idx_total, size_t pred, int num_sms,
                               bool clusters, int64_t listed) {
   const int64_t T1 = T > 0 ? T : 1;
   size_t most = 0;
-  for (int k = 0; k < 3; k++) {
+  for (int k = 0; k < 3; k++) {  // 128, 256 and 512 threads
     const int Mk = k < 2 ? std::min(M, kMixTop[k]) : M;
-    const int64_t G = std::min<int64_t>((int64_t)num_sms * (kScrThreads / mix_threads(Mk)), T1);
+    const int64_t G = std::min<int64_t>((int64_t)num_sms * (4 >> k), T1);
     most = std::max(most, mix_layout(G, p, n, mix_qpad(Mk, 1), idx_total, pred, listed).total);
   }
   for (int CL = 2; clusters && CL <= kMaxCL; CL *= 2) {

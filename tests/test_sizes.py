@@ -19,6 +19,7 @@ using namespace lagp;
 static int bad(const char *what, long a, long b, long c) { printf("%s %ld %ld %ld\n", what, a, b, c); return 1; }
 int main() {
   const int sms = 152;
+  const ScreenChip chip{sms, 132120576, 495616};
   const int Ms[] = {3, 64, 200, 256, 257, 500, 511, 512, 513, 600, 767, 768, 769, 800, 1000, 1023, 1024, 1025, 1100, 1343, 1344, 1345,
                     1500, 2000, 2047, 2048, 2049, 3000, 4096, 4097, 6000, 8192};
   const int ns[] = {3, 20, 50, 73, 100, 208, 209, 256};
@@ -33,7 +34,7 @@ int main() {
           if (a < prev) return bad("mix M", T, n, M);
           prev = a;
           // the grid of the shape that runs, whole, in what was asked for at this or any larger size
-          const int64_t G = std::min<int64_t>((int64_t)sms * (kScrThreads / mix_threads(M)), T);
+          const int64_t G = std::min<int64_t>((int64_t)sms * (kScrThreads / mix_threads(T, M, n, chip)), T);
           if (mix_fit(G, a, 8, n, mix_qpad(M, 1), T * n, 256, sms, 0) != G) return bad("mix fit", T, n, M);
           if (mix_asked_bytes(T + 1, 8, n, M, (T + 1) * n, 256, sms, c, 0) < a) return bad("mix T", T, n, M);
           if (n < 256 && M > n && mix_asked_bytes(T, 8, n + 1, M, T * (n + 1), 256, sms, c, 0) < a) return bad("mix n", T, n, M);
