@@ -23,13 +23,24 @@ __device__ __forceinline__ int tri_row(int e) {
   return a;
 }
 
+// a / l from q = rn(a r), r = rn(1 / l).  exact: also where the correction would leave the normal
+// range or meet an infinity (there it turns an infinite quotient into NaN), as a division.
+__device__ __forceinline__ double div_by_pivot(double a, double q, double l, double r, bool exact) {
+  if (exact) {
+    const unsigned ha = (unsigned)__double2hiint(a) & 0x7fffffffu, hq = (unsigned)__double2hiint(q) & 0x7fffffffu;
+    // both within 2^-960 .. 2^1023, or a = 0
+    if ((ha < (64u << 20) || hq < (64u << 20) || hq >= 0x7ff00000u) && (ha | (unsigned)__double2loint(a))) return a / l;
+  }
+  return fma(fma(-q, l, a), r, q);
+}
+
 // In-place Cholesky A = L L^T of the n x n lower triangle of A (row-major, leading
 // dimension lda), carrying naug extra columns n .. n+naug-1 along so that they end as
 // L^{-1} b (forward substitution).  rl[k] receives 1 / l_kk.  Sets *fail (shared) on a
 // pivot <= 0; every thread returns after the same barriers.
 // recip: the matrix entries (not the extra columns) are multiplied by 1 / l_kk instead of
-// divided by l_kk: the rounding of the FP64 recursion's candidate rows (select.cu), so a
-// design's rows come out bit for bit as that recursion forms them.
+// divided by l_kk, and the extra columns divided whatever their values: the rounding of the FP64
+// recursion (select.cu), so a design's rows come out bit for bit as that recursion forms them.
 // turn: the warp that takes the pivots.  Warp w of every CTA runs on sub-partition w mod 4, so
 // CTAs that share an SM should have them taken by different ones.
 __device__ void chol_flat_fp64(double *A, int n, int lda, int naug, double *rl, int *fail,
@@ -50,7 +61,7 @@ __device__ void chol_flat_fp64(double *A, int n, int lda, int naug, double *rl, 
     for (int i = k + 1 + tid; i < n + naug; i += nt) {
       double *ap = (i < n) ? &A[i * lda + k] : &A[k * lda + i];
       const double a = *ap, q = a * r;
-      *ap = (recip && i < n) ? q : fma(fma(-q, lkk, a), r, q);
+      *ap = (recip && i < n) ? q : div_by_pivot(a, q, lkk, r, recip);
     }
     __syncthreads();
     // a_il -= l_ik l_lk for k < l <= i, and the extra columns: b_i -= l_ik b_k

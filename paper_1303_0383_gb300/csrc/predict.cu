@@ -70,7 +70,7 @@ __device__ __forceinline__ bool pred_index_ok(const PredParams &P, const LocPara
   return LAGP_CHK(d[i], L.N, P.nn ? 24 : 41);
 }
 
-__global__ void __launch_bounds__(PB) predict_fp64_kernel(PredParams P) {
+__global__ void __launch_bounds__(PB, 10) predict_fp64_kernel(PredParams P) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nmax = P.nmax;
   double *rl = reinterpret_cast<double *>(smraw);     // nmax: 1 / l_kk
@@ -183,7 +183,7 @@ predict_group_kernel(PredParams P) {
         for (int i = k + 1 + t; i < n + 2; i += TT) {
           double *ap = i < n ? &A[i * (i + 1) / 2 + k] : &B[2 * k + i - n];
           const double a = *ap, q = a * r;
-          *ap = (P.recip && i < n) ? q : fma(fma(-q, lkk, a), r, q);
+          *ap = (P.recip && i < n) ? q : div_by_pivot(a, q, lkk, r, P.recip);
         }
       }
       __syncthreads();
