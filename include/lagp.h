@@ -331,9 +331,10 @@ int lagp_exp_dev(const double *x, double *y, int64_t n, void *stream);
  * location is abandoned.  Waits for the device, then returns in *count the violations since
  * the last call and in *site, *index, *bound the first one (site codes: 1-5 kernel (a):
  * survivor list, survivor design index, bucket scatter, bucket permutation, output index;
- * 11, 13-15, 18, 20 the mixed ALC screen: candidate design index, n, candidate count,
- * dimension, tensor-memory column, shared-memory layout; 21-25 the FP64 ALC kernel: n,
- * candidate count, dimension, candidate design index, shared-memory layout; 31-32 the
+ * 11-16, 18, 20 the ALC screen: candidate design index (mixed; 24 in FP64), candidate pair, n,
+ * candidate count, dimension, design rank, tensor-memory column, shared-memory layout; 21-25 the
+ * FP64 ALC kernel: n, candidate count, dimension, candidate design index, shared-memory layout; 24
+ * and 41 kernel (c): design index, of NN's candidates or of a given design; 31-32 the
  * paper-form kernel: candidate design index, shared-memory layout), and clears the records.
  * *checked = 1 in the checked build, 0 otherwise (where every count is 0).  Any output may
  * be NULL. */

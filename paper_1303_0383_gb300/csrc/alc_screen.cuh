@@ -78,10 +78,6 @@ __device__ __forceinline__ void tmem_wait16(uint32_t (&v)[16]) {
                :
                : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t ta, uint32_t (&v)[16]) {
-  tmem_ld16_issue(ta, v);
-  tmem_wait16(v);
-}
 __device__ __forceinline__ uint32_t as_word(float x) { return __float_as_uint(x); }
 __device__ __forceinline__ uint32_t as_word(int x) { return (uint32_t)x; }
 template <class Word>

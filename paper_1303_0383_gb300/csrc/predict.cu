@@ -89,8 +89,9 @@ __global__ void __launch_bounds__(PB, 10) predict_fp64_kernel(PredParams P) {
     const LocParams L = pred_loc(P, sh_loc);
     const int32_t *d = pred_design(P, L);
     if (tid < L.p) xl[tid] = L.x[tid];
-    bool ok = true;
-    for (int i = tid; i < L.n; i += PB) ok = ok && pred_index_ok(P, L, d, i);
+    bool ok = d[0] >= 0;  // (a failed location has no design: nothing to check)
+    if (ok)
+      for (int i = tid; i < L.n; i += PB) ok = ok && pred_index_ok(P, L, d, i);
     if (!__syncthreads_and(ok)) {
       if (tid == 0) predict_failed(L.loc, P.mean, P.s2, P.var, P.status);
       pred_idx_out(P, L, true, tid, PB);
