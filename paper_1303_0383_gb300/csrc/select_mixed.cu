@@ -46,6 +46,7 @@ namespace cg = cooperative_groups;
 struct FxFormat {
   int fmt[2];           // sh2b, e
   unsigned dmax, kmax;  // high words of the largest |x_c - x| and K(x, c)
+  int near;             // candidates with a K(x, c) within 2^-100 of the largest
   int odd;              // a coordinate is not finite
 };
 
@@ -89,11 +90,15 @@ struct MixParams {
 // from every candidate that cov^2 leaves FP64's normal range: there the recursion's scores lose bits
 // or tie at 0, and the screen's, scaled by the largest K(x, c) = 2^-w or more, do not.  cov shrinks
 // from 2^-w by 2^-53 at most before it is rounding error, and is compared as cov^2 v' with v' of
-// 2^-30 or more: 2 (w + 53) + 30 < 1022 for w <= 400.
+// 2^-30 or more: 2 (w + 53) + 30 < 1022 for w <= 400.  And fewer than 4 n / 5 candidates with a K(x, c)
+// within 2^-100 of the largest (small lengthscales): the later steps would be among candidates whose
+// scores are rounding error, a re-score of them all each.  (Emulated, 2000 points on a square of
+// side 4, n = 50 of 200, theta = 1e-3: 20 such steps at 20 candidates, 7 at 28, 0.7 at 36; none at 40 and theta
+// = 1.3e-3.)
 template <int MBT>
 __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, const double *etab, int4 *vp,
                                          int4 *cp, int4 *Xr, unsigned char *used, int Qpad, bool greedy, FxFormat &F) {
-  const int tid = threadIdx.x, p = L.p, M = L.M;
+  const int tid = threadIdx.x, p = L.p, M = L.M, n = L.n;
   long long *v = reinterpret_cast<long long *>(vp), *cov = reinterpret_cast<long long *>(cp);
   // e even with 1 + g < 2^(e+1)
   const int e = (ilogb(L.onepg) + 1) & ~1;
@@ -101,6 +106,7 @@ __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, c
   const double csc = sqrt(L.theta_inv * 1.4426950408889634);  // K = 2^-(squared distance) in these units
   if (tid == 0) {
     F.dmax = F.kmax = 0u;
+    F.near = 0;
     F.odd = !(csc >= 0.0 && csc < INFINITY);
   }
   __syncthreads();
@@ -144,10 +150,12 @@ __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, c
   const double fsc = scalbn(csc, 28 - b);
   const int w = min(max(1023 - (int)(F.kmax >> 20), 0), 1022);
   const double kw = scalbn(1.0, w), ke = scalbn(1.0, 59 - e);
+  int near = 0;
   for (int c = tid; c < 2 * Qpad; c += MBT) {
     const double kx = reinterpret_cast<double *>(cov)[c];
     const bool live = kx >= 0.0;
     cov[c] = live ? __double2ll_rn(kx * kw * ke) : 0;
+    near += kx * kw >= 0x1p-100;
     const double *xc = L.X + (live ? (int64_t)L.cand[c] * p : 0);
     for (int k = 0; k < p; k++) {
       const double f = live ? (xc[k] - xl[k]) * fsc : 0.0;
@@ -157,11 +165,28 @@ __device__ __noinline__ bool fx_location(const LocParams &L, const double *xl, c
       slot[2] = __double2int_rn((f - (double)xh) * 1073741824.0);  // 2^30
     }
   }
+  near = __reduce_add_sync(0xffffffffu, near);
+  if ((tid & 31) == 0) atomicAdd(&F.near, near);
   if (tid == 0) {
     F.fmt[0] = min(2 * b, 62);
     F.fmt[1] = e;
   }
-  return b > 8 || F.odd || (greedy && w > 400);
+  __syncthreads();
+  return b > 8 || F.odd || (greedy && (w > 400 || 5 * F.near < 4 * n));
+}
+
+// FxArith: whether a location is better left to the FP64 recursion after re-scores of weight m / 8 (8 and
+// one per candidate each) in `steps` greedy steps, at a design of j + 1 points: if they go on at that
+// pace, they take more than half as long as the recursion.  A pass rebuilds the design's factor, a
+// chain of about 3.2 us per column; the recursion takes 8 us a step and 0.25 ns more per candidate
+// and (n + 60) (GB300, 300 locations, n = 50 and 100, M = 200 to 2000).  Designs without such structure
+// re-score 0 to 2 times in 44 steps.  Whole calls, the recursion alone, every re-score made, this
+// rule: near-duplicate points, n = 50 of 200 0.65, 4.28, 0.80 ms, n = 100 of 400 2.49, 27.9, 2.76; theta =
+// 1e-3, n = 50 of 1000 1.77, 261, 1.85.
+__device__ __forceinline__ bool rescore_pace(int m, int steps, int j, int n, int M) {
+  const float rest = 0.2f * (float)(n * n - j * j) * (float)m / (float)steps;
+  const float all = (float)n * (8.0f + (float)M * (float)(n + 60) * 2.5e-4f);
+  return m >= 24 && 2.0f * rest > all;
 }
 
 // MBT threads per CTA, one location per CTA, one or two candidate pairs per thread up to 1024
@@ -202,7 +227,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
   __shared__ int xr_r[CLU ? kMaxCL : 1];
   __shared__ double red_n[NWARP], red_d[NWARP];
   __shared__ int red_rr[NWARP];
-  __shared__ int sh_loc, sh_fail, sh_nlist, sh_per;
+  __shared__ int sh_loc, sh_fail, sh_nlist, sh_per, sh_passes;
   __shared__ LocParams L;  // the location's parameters: read where they are used
   __shared__ FxFormat fx;                // the location's formats (FxArith)
   __shared__ unsigned sh_top[3], sh_nwr[3];  // by step: best score key of the warps that are done,
@@ -296,7 +321,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       continue;
     if (tid < p) xl[tid] = L.x[tid];
     if (tid == 0) {
-      sh_fail = 0;
+      sh_fail = sh_passes = 0;
       // a last round of up to 64 pairs would leave nearly all threads idle for its row loops' latency:
       // rounds of like size then (600 8-d locations, n = 100 of 2100: 11.3 -> 10.3 ms; a larger rest is
       // better on its own)
@@ -518,6 +543,12 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       int br;
       rescore_fp64<A>(R, B1, &bn, &bd, &br);
       if (sh_fail) break;  // the same in every CTA of a cluster
+      if constexpr (A::kFixed) {
+        __syncthreads();  // (every thread has read sh_fail)
+        if (tid == 0 && rescore_pace(sh_passes += 8 + sh_nlist, j + 2 - n0e, j, n, M)) sh_fail = 1;
+        __syncthreads();
+        if (sh_fail) break;
+      }
       if constexpr (CLU) {  // the cluster's FP64 best, ties to the nearer candidate
         cg::cluster_group cl = cg::this_cluster();
         if (tid == 0)
