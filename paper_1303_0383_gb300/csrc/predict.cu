@@ -12,7 +12,7 @@
 // line: packed triangles of one location and of the index table fill the 227 KB).
 // GB300, NN's 3000 locations, one-location kernel or the recursion before -> groups: n = 50
 // 2.65 -> 0.45 ms, n = 100 7.74 -> 1.95, n = 180 20.8 -> 12.7, n = 208 27.5 -> 18.1 (one-location
-// kernel at n = 209: 24.8); one location: n = 50 267 -> 69 us, n = 208 2.40 -> 0.91 ms.
+// kernel at n = 209, 128 threads: 24.8); one location: n = 50 267 -> 69 us, n = 208 2.40 -> 0.91 ms.
 #include <math.h>
 
 #include "check.cuh"
@@ -21,7 +21,7 @@
 namespace lagp {
 namespace {
 
-constexpr int PB = 128;              // threads per CTA of the one-location kernel
+constexpr int PB = 512;              // threads per CTA of the one-location kernel
 constexpr int kMaxGroup = 8;         // locations of a group
 constexpr int kGroupMaxN = 208;      // largest n of the group kernel
 constexpr size_t kGroupSmem = 112 * 1024;  // two CTAs per SM where a group of two or more fits
@@ -70,7 +70,11 @@ __device__ __forceinline__ bool pred_index_ok(const PredParams &P, const LocPara
   return LAGP_CHK(d[i], L.N, P.nn ? 24 : 41);
 }
 
-__global__ void __launch_bounds__(PB, 10) predict_fp64_kernel(PredParams P) {
+// One location in 512 threads: each column's update is n^2 / 2 entries behind two block barriers, and
+// 128 threads took 110 rounds of loads from L2 for it at n = 256.  GB300, 128 -> 512 threads: n = 220
+// one location 5.12 -> 1.51 ms, 600 9.71 -> 4.59, 3000 29.7 -> 22.0; n = 256 8.67 -> 2.46, 16.3 -> 7.26,
+// 46.1 -> 34.4.
+__global__ void __launch_bounds__(PB, 2) predict_fp64_kernel(PredParams P) {
   extern __shared__ __align__(16) unsigned char smraw[];
   const int nmax = P.nmax;
   double *rl = reinterpret_cast<double *>(smraw);     // nmax: 1 / l_kk
@@ -250,9 +254,9 @@ int pred_grid(int64_t T, int nmax, const DevInfo &di) {
 }
 
 // Worst-case grid for sizing the workspace before the occupancy is known: at most this many
-// CTAs of 128 threads per SM (2048 threads per SM).
+// CTAs of 512 threads per SM (2048 threads per SM).
 int pred_grid_bound(int64_t T, int num_sms) {
-  const int64_t g = (int64_t)num_sms * 16;
+  const int64_t g = (int64_t)num_sms * (2048 / PB);
   return (int)(T < g ? (T > 0 ? T : 1) : g);
 }
 
