@@ -32,6 +32,8 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include <algorithm>
+
 #include "alc_screen.cuh"
 #include "batch.cuh"
 #include "check.cuh"
@@ -667,15 +669,17 @@ MixVariant mix_variant(int64_t T, int M, int n, int CL, bool fixed, const DevInf
   return MixVariant{threads, mix_qpad(M, 1) <= 128 ? 1 : 2, 1, fixed};
 }
 
+// A CTA's share of an SM's shared memory, without what it takes besides (static, 1 KB reserved).
+size_t mix_share(MixVariant v, const DevInfo &di) {
+  return std::min(di.smem_per_sm / mix_minb(v), di.smem_optin + 1024) - (mix_static_smem(v) + 1024);
+}
+
 // Records and dynamic shared memory of a launch whose largest location has Qpad pairs and n
 // points: a CTA takes its whole share of the SM, the factor rows filling what the state leaves
 // (row i is read at every step after step i, so the first rows carry the most traffic; the
 // rest stream from tensor memory and L2); a state larger than the share takes what it needs.
 void mix_smem(int Qpad, int n, MixVariant v, const DevInfo &di, int *nrec, size_t *smem) {
-  const size_t over = mix_static_smem(v) + 1024;  // 1 KB reserved per CTA
-  size_t share = di.smem_per_sm / mix_minb(v);
-  if (share > di.smem_optin + 1024) share = di.smem_optin + 1024;
-  share -= over;
+  const size_t share = mix_share(v, di);
   *nrec = v.CL > 1 ? 1 : kRecords;
   while (*nrec > 1 && mix_state_bytes(Qpad, n, *nrec, v) > share) --*nrec;
   const size_t need = mix_state_bytes(Qpad, n, *nrec, v);
@@ -756,11 +760,19 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, size_
   if (st) return st;
   cudaError_t e;
   if (v.CL == 1) {
-    // every resident CTA holds its share of the SM's 512 tensor-memory columns; 128 registers
-    // per thread keep the residents at kScrThreads, so an allocation never waits
+    // every resident CTA holds its share of the SM's 512 tensor-memory columns, and an allocation
+    // must never wait: no more than mix_minb CTAs may be resident.  Their registers see to it
+    // unless the compiler needs fewer than the 128 it may take; then the CTA's whole share of
+    // shared memory, of which one more would not find any left, does
     int k = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, mix_kernel(v), v.MBT, smem);
     if (e != cudaSuccess) return cuda_status(e);
+    if (k > mix_minb(v)) {
+      smem = std::max(smem, mix_share(v, di));
+      P.smem = (int)smem;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, mix_kernel(v), v.MBT, smem);
+      if (e != cudaSuccess) return cuda_status(e);
+    }
     if (k * tmem_cols(v.MBT) > 512) return LAGP_ERR_CUDA;
   }
   e = cudaMemsetAsync(w, 0, 512, stream);  // the counters
