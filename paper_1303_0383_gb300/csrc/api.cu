@@ -6,6 +6,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 
@@ -319,10 +320,16 @@ int lagp_predict_dev(const double *X, const double *Z, int64_t N, int32_t p, con
   if (T == 0) return LAGP_OK;
   if (!X || !Z || !XX || !mean || !s2 || !workspace) return LAGP_ERR_INVALID_ARG;
   if (((uintptr_t)workspace & 255) != 0) return LAGP_ERR_INVALID_ARG;
-  if (workspace_bytes < lagp_predict_workspace_bytes(N, T, p, n, ncand, method, precision))
+  // (less than was asked for: the candidate search without its scan, smaller grids)
+  DevInfo di;
+  st = dev_info(&di);
+  if (st) return st;
+  SelectArgs a = {};
+  a.p = p; a.T = T; a.M = ncand; a.n0 = n0; a.n = n; a.g = g; a.method = method; a.precision = precision;
+  size_t cand_bytes = align_up((size_t)T * (size_t)ncand * sizeof(int32_t), 256);
+  if (workspace_bytes < cand_bytes + std::max(knn_base_bytes(N), select_needed_bytes(a, di.num_sms)))
     return LAGP_ERR_INVALID_ARG;
   char *w = static_cast<char *>(workspace);
-  size_t cand_bytes = align_up((size_t)T * (size_t)ncand * sizeof(int32_t), 256);
   int32_t *cand = reinterpret_cast<int32_t *>(w);
   void *rest = w + cand_bytes;
   size_t rest_bytes = workspace_bytes - cand_bytes;

@@ -120,6 +120,7 @@ BatchLayout layout_of(const BatchPlan &P, int32_t method, int32_t precision, int
   BatchLaunch b = make_launch(P, method, precision, T, nullptr, 0, nullptr, nullptr, nullptr,
                               nullptr, nullptr, select_max_ctas(method, precision));
   L.sel_ws = select_batch_workspace_bytes(b, num_sms);
+  L.sel_needed = select_batch_needed_bytes(b, num_sms);
   L.total = L.scratch + std::max(L.knn_ws, L.sel_ws);
   return L;
 }
@@ -201,14 +202,13 @@ cudaStream_t capture_stream(int device) {
 static int launch_all(const BatchPlan &P, const BatchLayout &L, char *w, const double *XX, int32_t ldxx,
                       int64_t T, int32_t method, int32_t precision, double *mean, double *s2,
                       double *var, int32_t *idx, int8_t *status, int knn_ctas, int sel_ctas,
-                      cudaStream_t stream) {
+                      size_t sbytes, cudaStream_t stream) {
   const BatchDesign *ddev = reinterpret_cast<const BatchDesign *>(w + L.designs);
   const LocDesc *ldev = reinterpret_cast<const LocDesc *>(w + L.locs);
   const int32_t *odev = reinterpret_cast<const int32_t *>(w + L.order);
   const int32_t *lsdev = reinterpret_cast<const int32_t *>(w + L.lists);
   int32_t *cand = reinterpret_cast<int32_t *>(w + L.cand);
   void *scratch = w + L.scratch;
-  const size_t sbytes = std::max(L.knn_ws, L.sel_ws);
   for (size_t d = 0; d < P.designs.size(); d++) {
     const int cnt = P.list_cnt[d];
     if (!cnt) continue;
@@ -257,7 +257,9 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
   st = dev_info(&di);
   if (st) return st;
   const BatchLayout L = layout_of(P, method, precision, T, di.num_sms);
-  if (workspace_bytes < L.total) return LAGP_ERR_INVALID_ARG;
+  // (less than was asked for: the candidate search without its scan, smaller grids)
+  if (workspace_bytes < L.scratch + std::max(knn_base_bytes(P.Nmax), L.sel_needed)) return LAGP_ERR_INVALID_ARG;
+  const size_t sbytes = workspace_bytes - L.scratch;
   cudaStream_t stream = static_cast<cudaStream_t>(stream_);
   char *w = static_cast<char *>(workspace);
   // tables to the device (outside any graph: the host vectors are pageable)
@@ -295,7 +297,7 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
       for (int so = 1; so <= smax; so++) {
         cudaEventRecord(e0, stream);
         st = launch_all(P, L, w, XX, ldxx, T, method, precision, mean, s2, var, idx, status,
-                        kn_opts[ko], so, stream);
+                        kn_opts[ko], so, sbytes, stream);
         cudaEventRecord(e1, stream);
         if (st) break;
         if (cudaEventSynchronize(e1) != cudaSuccess) { st = LAGP_ERR_CUDA; break; }
@@ -343,7 +345,7 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
       if (e != cudaSuccess) return cuda_status(e);
       const int64_t before = g_launches.load();
       st = launch_all(P, L, w, XX, ldxx, T, method, precision, mean, s2, var, idx, status,
-                      knn_ctas, sel_ctas, cap);
+                      knn_ctas, sel_ctas, sbytes, cap);
       g->kernels = g_launches.load() - before;
       g_launches.fetch_sub(g->kernels);  // recorded, not run
       e = cudaStreamEndCapture(cap, &graph);
@@ -359,5 +361,5 @@ extern "C" int lagp_predict_batch_dev(const lagp_design_desc *designs, int32_t n
     return cuda_status(e);
   }
   return launch_all(P, L, w, XX, ldxx, T, method, precision, mean, s2, var, idx, status, knn_ctas,
-                    sel_ctas, stream);
+                    sel_ctas, sbytes, stream);
 }

@@ -29,7 +29,7 @@ struct LocDesc {
 
 struct BatchLayout {
   size_t designs, locs, order, lists, cand, scratch, total;
-  size_t knn_ws, sel_ws;
+  size_t knn_ws, sel_ws, sel_needed;
 };
 
 struct BatchPlan {
@@ -74,7 +74,7 @@ inline std::string batch_graph_key(const BatchPlan &P, const BatchLayout &L, con
   put(P.nmax), put(P.pmax), put(P.Mmax), put(P.Nmax), put(P.cand_total), put(P.idx_total);
   put(P.gmin());  // chooses the FP64 form
   put(L.designs), put(L.locs), put(L.order), put(L.lists), put(L.cand), put(L.scratch), put(L.total);
-  put(L.knn_ws), put(L.sel_ws);
+  put(L.knn_ws), put(L.sel_ws), put(L.sel_needed);
   for (size_t d = 0; d < P.designs.size(); d++) {
     const BatchDesign &D = P.designs[d];
     put(D.X), put(D.Z), put(D.N), put(D.p);

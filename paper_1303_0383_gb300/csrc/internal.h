@@ -63,6 +63,8 @@ struct SelectArgs {
 size_t select_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int32_t method,
                               int32_t precision, int num_sms);
 int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream);
+// The least workspace that select_launch takes (one CTA per SM, or the FP64 recursion).
+size_t select_needed_bytes(const SelectArgs &a, int num_sms);
 // The same launch on a caller-chosen grid of G CTAs (G >= 1), and the scratch it needs.
 int select_default_grid(int64_t T, int num_sms);
 size_t select_scratch_bytes_for_grid(int G, int32_t p, int32_t n, int32_t ncand);
@@ -81,7 +83,7 @@ int select_listed_launch(const SelectArgs *a, const BatchLaunch *b, const Handed
 
 // Mixed-precision variant of kernels (b)+(c) (ALC): float-float screen, FP64 decisions.
 size_t select_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int32_t precision, int num_sms);
-bool select_mixed_fits(const SelectArgs &a, size_t ws_bytes);  // room for one CTA per SM at least
+size_t select_mixed_needed_bytes(const SelectArgs &a);  // room for one CTA per SM
 int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream);
 
 // ALC in the paper's own form (explicit K_j^{-1}, partition inverse updates), FP64:
@@ -136,6 +138,7 @@ int mle_prepare();
 
 // MSPE variant of kernels (b)+(c), FP64.
 size_t select_mspe_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms);
+size_t select_mspe_needed_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms);
 int select_mspe_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream);
 // MSPE, mixed precision: float-float screen, FP64 bookkeeping and decisions.
 size_t select_mspe_mixed_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms);
@@ -171,8 +174,9 @@ int select_mspe_prepare();
 int select_mspe_mixed_prepare();
 size_t select_batch_workspace_bytes(const BatchLaunch &b, int num_sms);
 int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream);
+size_t select_batch_needed_bytes(const BatchLaunch &b, int num_sms);
 size_t select_mixed_batch_workspace_bytes(const BatchLaunch &b);
-bool select_mixed_batch_fits(const BatchLaunch &b, size_t ws_bytes);
+size_t select_mixed_batch_needed_bytes(const BatchLaunch &b);
 int select_mixed_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream);
 size_t select_mspe_batch_workspace_bytes(const BatchLaunch &b, int G);
 int select_mspe_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, int G, cudaStream_t stream);

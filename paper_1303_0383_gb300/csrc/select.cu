@@ -312,6 +312,16 @@ static PredictArgs nn_args(const double *XX, int64_t T, int n, const int32_t *ca
   return pa;
 }
 
+size_t select_needed_bytes(const SelectArgs &a, int num_sms) {
+  if (a.method == LAGP_MSPE)
+    return a.precision == LAGP_MIXED ? select_mspe_mixed_workspace_bytes(a.T, a.p, a.n, a.M, num_sms)
+                                     : select_mspe_needed_bytes(a.T, a.p, a.n, a.M, num_sms);
+  const size_t own = select_scratch_bytes_for_grid(sel_grid(a.T, num_sms), a.p, a.n, a.M);
+  if (a.method == LAGP_NN) return std::min(own, predict_fp64_workspace_bytes(a.T, a.n, num_sms));
+  const size_t scr = select_mixed_needed_bytes(a);
+  return a.precision == LAGP_MIXED ? scr : screened(a.method, a.g, a.r_min) ? std::min(own, scr) : own;
+}
+
 int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
   if (a.T == 0) return LAGP_OK;
   if (a.method == LAGP_MSPE)
@@ -324,7 +334,7 @@ int select_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t s
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  if (screened(a.method, a.g, a.r_min) && select_mixed_fits(a, ws_bytes))
+  if (screened(a.method, a.g, a.r_min) && ws_bytes >= select_mixed_needed_bytes(a))
     return select_mixed_launch(a, ws, ws_bytes, stream);
   if (a.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(a.T, a.n, di.num_sms)) {
     PredictArgs pa = nn_args(a.XX, a.T, a.n, a.cand, a.M, a.mean, a.s2, a.var, a.idx, a.status);
@@ -436,6 +446,17 @@ size_t select_batch_workspace_bytes(const BatchLaunch &b, int num_sms) {
   return b.precision == LAGP_MIXED || scr > own ? scr : own;
 }
 
+size_t select_batch_needed_bytes(const BatchLaunch &b, int num_sms) {
+  const int G = batch_grid(b, num_sms);
+  if (b.method == LAGP_MSPE)
+    return b.precision == LAGP_MIXED ? select_mspe_mixed_batch_workspace_bytes(b, G)
+                                     : select_mspe_batch_workspace_bytes(b, std::min(G, num_sms));
+  const size_t own = select_scratch_bytes_for_grid(G, b.pmax, b.nmax, b.Mmax);
+  if (b.method == LAGP_NN) return std::min(own, predict_fp64_workspace_bytes(b.T, b.nmax, num_sms));
+  const size_t scr = select_mixed_batch_needed_bytes(b);
+  return b.precision == LAGP_MIXED ? scr : screened(b.method, b.gmin, 0.0) ? std::min(own, scr) : own;
+}
+
 int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStream_t stream) {
   if (b.T == 0) return LAGP_OK;
   DevInfo di;
@@ -443,12 +464,14 @@ int select_batch_launch(const BatchLaunch &b, void *ws, size_t ws_bytes, cudaStr
   if (st) return st;
   st = exp_table_upload();
   if (st) return st;
-  const int G = batch_grid(b, di.num_sms);
-  if (b.method == LAGP_MSPE)
-    return b.precision == LAGP_MIXED ? select_mspe_mixed_batch_launch(b, ws, ws_bytes, G, stream)
-                                     : select_mspe_batch_launch(b, ws, ws_bytes, G, stream);
+  int G = batch_grid(b, di.num_sms);
+  if (b.method == LAGP_MSPE) {
+    if (b.precision == LAGP_MIXED) return select_mspe_mixed_batch_launch(b, ws, ws_bytes, G, stream);
+    if (ws_bytes < select_mspe_batch_workspace_bytes(b, G)) G = std::min(G, di.num_sms);  // one CTA per SM
+    return select_mspe_batch_launch(b, ws, ws_bytes, G, stream);
+  }
   if ((b.precision == LAGP_MIXED && b.method == LAGP_ALC) ||
-      (screened(b.method, b.gmin, 0.0) && select_mixed_batch_fits(b, ws_bytes)))
+      (screened(b.method, b.gmin, 0.0) && ws_bytes >= select_mixed_batch_needed_bytes(b)))
     return select_mixed_batch_launch(b, ws, ws_bytes, stream);
   if (b.method == LAGP_NN && ws_bytes >= predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms)) {
     PredictArgs pa = nn_args(b.XX, b.T, b.nmax, b.cand, b.Mmax, b.mean, b.s2, b.var, b.idx, b.status);

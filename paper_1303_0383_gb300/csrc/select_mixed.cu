@@ -826,10 +826,15 @@ static int mix_uniform_fit(const SelectArgs &a, MixVariant v, size_t ws_bytes, c
                  predict_fp64_workspace_bytes(a.T, a.n, di.num_sms), di.num_sms, v.fixed ? a.T : 0);
 }
 
-bool select_mixed_fits(const SelectArgs &a, size_t ws_bytes) {
+size_t select_mixed_needed_bytes(const SelectArgs &a) {
   DevInfo di;
-  return dev_info(&di) == LAGP_OK && mix_uniform_fit(a, mix_variant(a.T, a.M, a.n, 1, a.precision == LAGP_FP64, di), ws_bytes,
-                                                       di) > 0;
+  if (dev_info(&di)) return SIZE_MAX;
+  const bool fixed = a.precision == LAGP_FP64;
+  const MixVariant v = mix_variant(a.T, a.M, a.n, fixed ? 1 : mix_cluster_size(), fixed, di);
+  if (v.CL > 1) return select_mixed_workspace_bytes(a.T, a.p, a.n, a.M, a.precision, di.num_sms);
+  const int64_t G = std::min<int64_t>(mix_grid(a.T, di.num_sms, v), di.num_sms);
+  return mix_layout(G, a.p, a.n, mix_qpad(a.M, 1), a.T * a.n, predict_fp64_workspace_bytes(a.T, a.n, di.num_sms),
+                    fixed ? a.T : 0).total;
 }
 
 int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
@@ -881,9 +886,12 @@ static int mix_batch_fit(const BatchLaunch &b, size_t ws_bytes, const DevInfo &d
                  b.precision == LAGP_FP64 ? b.T : 0);
 }
 
-bool select_mixed_batch_fits(const BatchLaunch &b, size_t ws_bytes) {
+size_t select_mixed_batch_needed_bytes(const BatchLaunch &b) {
   DevInfo di;
-  return dev_info(&di) == LAGP_OK && mix_batch_fit(b, ws_bytes, di) > 0;
+  if (dev_info(&di)) return SIZE_MAX;
+  const int64_t G = std::min<int64_t>(mix_batch_grid(b, di), di.num_sms);
+  return mix_layout(G, b.pmax, b.nmax, mix_qpad(b.Mmax, 1), b.idx_total,
+                    predict_fp64_workspace_bytes(b.T, b.nmax, di.num_sms), b.precision == LAGP_FP64 ? b.T : 0).total;
 }
 
 // (Locations grouped by candidate count, one launch of a fitting instance each, measured slower:

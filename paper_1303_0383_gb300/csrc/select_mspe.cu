@@ -462,6 +462,11 @@ size_t select_mspe_workspace_bytes(int64_t T, int32_t p, int32_t n, int32_t ncan
   return mspe_layout(mspe_grid(T, num_sms), p, n, ncand, T, T * n, num_sms).total;
 }
 
+// (one CTA per SM)
+size_t select_mspe_needed_bytes(int64_t T, int32_t p, int32_t n, int32_t ncand, int num_sms) {
+  return mspe_layout((int)(T < num_sms ? (T > 0 ? T : 1) : num_sms), p, n, ncand, T, T * n, num_sms).total;
+}
+
 int select_mspe_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStream_t stream) {
   if (a.T == 0) return LAGP_OK;
   DevInfo di;
