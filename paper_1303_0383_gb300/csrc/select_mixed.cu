@@ -663,9 +663,9 @@ int mix_cluster_size() {
   return e == 1 || e == 2 || e == 4 || e == 8 ? e : 1;
 }
 
-MixVariant mix_variant(int64_t T, int M, int n, int CL, bool fixed, const DevInfo &di) {
+MixVariant mix_variant(int64_t T, int M, int n, int p, int CL, bool fixed, const DevInfo &di) {
   if (CL > 1) return MixVariant{256, 2, CL, false};
-  const int threads = mix_threads(T, M, n, ScreenChip{di.num_sms, di.l2, di.smem_per_sm + kTmemBytes});
+  const int threads = mix_threads(T, M, n, p, ScreenChip{di.num_sms, di.l2, di.smem_per_sm + kTmemBytes});
   return MixVariant{threads, mix_qpad(M, 1) <= 128 ? 1 : 2, 1, fixed};
 }
 
@@ -801,7 +801,7 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, size_
 // A batch's instance suits its largest candidate count; the grid is the batch's share of
 // select_max_ctas() CTAs per SM, of that instance's residents.
 MixVariant mix_batch_variant(const BatchLaunch &b, const DevInfo &di) {
-  return mix_variant(b.T, b.Mmax, b.nmax, 1, b.precision == LAGP_FP64, di);
+  return mix_variant(b.T, b.Mmax, b.nmax, b.pmax, 1, b.precision == LAGP_FP64, di);
 }
 int mix_batch_grid(const BatchLaunch &b, const DevInfo &di) {
   const int most = select_max_ctas(b.method, b.precision);
@@ -830,7 +830,7 @@ size_t select_mixed_needed_bytes(const SelectArgs &a) {
   DevInfo di;
   if (dev_info(&di)) return SIZE_MAX;
   const bool fixed = a.precision == LAGP_FP64;
-  const MixVariant v = mix_variant(a.T, a.M, a.n, fixed ? 1 : mix_cluster_size(), fixed, di);
+  const MixVariant v = mix_variant(a.T, a.M, a.n, a.p, fixed ? 1 : mix_cluster_size(), fixed, di);
   if (v.CL > 1) return select_mixed_workspace_bytes(a.T, a.p, a.n, a.M, a.precision, di.num_sms);
   const int64_t G = std::min<int64_t>(mix_grid(a.T, di.num_sms, v), di.num_sms);
   return mix_layout(G, a.p, a.n, mix_qpad(a.M, 1), a.T * a.n, predict_fp64_workspace_bytes(a.T, a.n, di.num_sms),
@@ -845,7 +845,7 @@ int select_mixed_launch(const SelectArgs &a, void *ws, size_t ws_bytes, cudaStre
   st = exp_table_upload();
   if (st) return st;
   const bool fixed = a.precision == LAGP_FP64;
-  const MixVariant v = mix_variant(a.T, a.M, a.n, fixed ? 1 : mix_cluster_size(), fixed, di);
+  const MixVariant v = mix_variant(a.T, a.M, a.n, a.p, fixed ? 1 : mix_cluster_size(), fixed, di);
   const int Qpad = mix_qpad(a.M, v.CL);
   int G = mix_grid(a.T, di.num_sms, v);
   if (v.CL > 1) {

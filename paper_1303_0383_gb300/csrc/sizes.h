@@ -37,19 +37,20 @@ struct ScreenChip {
 // thread, 512 threads per SM in all.  Small CTAs leave fewer threads idle and hide each other's
 // barriers; large ones have a location to themselves sooner and keep fewer factor rows live.  So
 // CTAs of 128 and 256 threads are taken for up to 512 and 1024 candidates, and for half as many again
-// where more than two locations per SM are asked for and the rows of those in flight stay within L2
-// and the chip; with two per SM or fewer, 256 threads from 257 candidates on.  GB300, mixed, 2000 2-d
+// where more than two locations per SM are asked for and the rows and coordinates of those in
+// flight stay within nine tenths of L2 and the chip; with two per SM or fewer, 256 threads from 257
+// candidates on.  GB300, mixed, 2000 2-d
 // locations, n = 50, in ms for 128 / 256 / 512 threads: M = 400 1.50 / 1.79 / 2.51, 600 2.21 / 2.26 /
 // 3.17, 700 2.25 / 2.53 / 3.22, 1024 3.04 / 2.73 / 3.44, 1100 4.36 / 3.64 / 4.19, 1300 5.07 / 4.06 / 4.39,
 // 1500 5.72 / 4.72 / 4.42; 300 locations, M = 400 0.44 / 0.40 / 0.44; one, 0.27 / 0.24 / 0.24, M = 1100
 // 0.63 / 0.46 / 0.36; 600 8-d ones, n = 100: M = 300 1.67 / 2.08 / 2.48, 500 2.86 / 2.13 / 2.72, 1030 6.54 /
-// 5.67 / 4.23 (rows beyond L2).  kMixTop: the largest M of the first two.
+// 5.67 / 4.23 (rows beyond L2); n = 60, M = 700 1.52 / 1.31 (just beyond the line).  kMixTop: the largest M of the first two.
 constexpr int kMixTop[2] = {768, 1344};
-inline int mix_threads(int64_t T, int M, int n, const ScreenChip &c) {
+inline int mix_threads(int64_t T, int M, int n, int p, const ScreenChip &c) {
   const int Qpad = mix_qpad(M, 1);
   const bool many = T > 2 * (int64_t)c.num_sms;
-  const double room = (double)c.l2 + (double)c.num_sms * c.on_chip;
-  auto fits = [&](int k) { return 16.0 * k * c.num_sms * n * Qpad <= room; };  // k locations per SM
+  const double room = 0.9 * ((double)c.l2 + (double)c.num_sms * c.on_chip);
+  auto fits = [&](int k) { return 16.0 * k * c.num_sms * (n + p) * Qpad <= room; };  // k locations per SM
   if (Qpad <= 128 || (many && 2 * Qpad <= kMixTop[0] && fits(4))) return 128;
   if (2 * Qpad <= 1024 || (many && 2 * Qpad <= kMixTop[1] && fits(2))) return 256;
   return 512;

@@ -34,7 +34,7 @@ int main() {
           if (a < prev) return bad("mix M", T, n, M);
           prev = a;
           // the grid of the shape that runs, whole, in what was asked for at this or any larger size
-          const int64_t G = std::min<int64_t>((int64_t)sms * (kScrThreads / mix_threads(T, M, n, chip)), T);
+          const int64_t G = std::min<int64_t>((int64_t)sms * (kScrThreads / mix_threads(T, M, n, 8, chip)), T);
           if (mix_fit(G, a, 8, n, mix_qpad(M, 1), T * n, 256, sms, 0) != G) return bad("mix fit", T, n, M);
           if (mix_asked_bytes(T + 1, 8, n, M, (T + 1) * n, 256, sms, c, 0) < a) return bad("mix T", T, n, M);
           if (n < 256 && M > n && mix_asked_bytes(T, 8, n + 1, M, T * (n + 1), 256, sms, c, 0) < a) return bad("mix n", T, n, M);
