@@ -326,9 +326,9 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       sh_fail = sh_passes = 0;
       // a last round of up to 64 pairs would leave nearly all threads idle for its row loops' latency:
       // rounds of like size then (600 8-d locations, n = 100 of 2100: 11.3 -> 10.3 ms; a larger rest is
-      // better on its own)
+      // better on its own; CTAs of fewer threads take none that large)
       const int full = NP * MBT, q32 = (Qs + 31) & ~31, rest = q32 % full, rounds = (q32 + full - 1) / full;
-      sh_per = MBT == 512 && q32 > full && rest > 0 && rest <= 64 ? ((q32 + rounds - 1) / rounds + 31) & ~31 : full;
+      sh_per = q32 > full && rest > 0 && rest <= 64 ? ((q32 + rounds - 1) / rounds + 31) & ~31 : full;
     }
     __syncthreads();
     bool hand = false;  // (FxArith) the location is left to the FP64 recursion
@@ -449,10 +449,17 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       // multiple of 32 (all within Qpad; those past Qs only update state nobody reads), each
       // round's in two halves of whole warps
       const int Q32 = (Qs + 31) & ~31;
-      const int per = sh_per;  // pairs of a round
-      for (int base = 0, k = 0; base < Q32; base += per, k += NP) {
-        const int left = min(per, Q32 - base), dq = NP == 1 ? MBT : min(MBT, ((left >> 1) + 31) & ~31);
-        if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, base + tid, b1, r1, b2, k, tid + dq < left ? dq : 0);
+      if constexpr (MBT == 512) {
+        const int per = sh_per;  // pairs of a round
+        for (int base = 0, k = 0; base < Q32; base += per, k += NP) {
+          const int left = min(per, Q32 - base), dq = min(MBT, ((left >> 1) + 31) & ~31);
+          if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, base + tid, b1, r1, b2, k, tid + dq < left ? dq : 0);
+        }
+      } else {
+        for (int q = tid, k = 0; q - tid < Q32; q += NP * MBT, k += NP) {
+          const int left = Q32 - (q - tid), dq = NP == 1 ? MBT : min(MBT, ((left >> 1) + 31) & ~31);
+          if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, q, b1, r1, b2, k, q + dq < Q32 ? dq : 0);
+        }
       }
       // best and second-best screen scores of the warp; the warp writes the record of its own
       // best candidate as the next step's pivot before the barrier, so that the gather of the
@@ -547,7 +554,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       if (sh_fail) break;  // the same in every CTA of a cluster
       if constexpr (A::kFixed) {
         __syncthreads();  // (every thread has read sh_fail)
-        if (tid == 0 && rescore_pace(sh_passes += 8 + sh_nlist, j + 2 - n0e, j, n, M)) sh_fail = 1;
+        if (tid == 0 && rescore_pace(sh_passes += 8 + sh_nlist, j + 2 - n0e, j, L.n, L.M)) sh_fail = 1;
         __syncthreads();
         if (sh_fail) break;
       }
@@ -582,7 +589,7 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
     // evaluates the predictive equations on it in FP64.  (FxArith: whatever stopped the screen, the
     // recursion decides whether the location fails.)
     if constexpr (A::kFixed)
-      if (sh_fail && tid == 0) P.list[atomicAdd(P.nlist, 1)] = qloc;
+      if (sh_fail && tid == 0) P.list[atomicAdd(P.nlist, 1)] = sh_loc;  // (its queue position)
     if (crank == 0) {
       for (int i = tid; i < n; i += MBT)
         L.idx[i] = (sh_fail || i >= ne || !LAGP_CHK(dr[i], M, 16)) ? -1 : L.cand[dr[i]];
