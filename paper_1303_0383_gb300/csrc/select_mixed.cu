@@ -326,9 +326,9 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       sh_fail = sh_passes = 0;
       // a last round of up to 64 pairs would leave nearly all threads idle for its row loops' latency:
       // rounds of like size then (600 8-d locations, n = 100 of 2100: 11.3 -> 10.3 ms; a larger rest is
-      // better on its own; CTAs of fewer threads take none that large)
+      // better on its own)
       const int full = NP * MBT, q32 = (Qs + 31) & ~31, rest = q32 % full, rounds = (q32 + full - 1) / full;
-      sh_per = q32 > full && rest > 0 && rest <= 64 ? ((q32 + rounds - 1) / rounds + 31) & ~31 : full;
+      sh_per = MBT == 512 && q32 > full && rest > 0 && rest <= 64 ? ((q32 + rounds - 1) / rounds + 31) & ~31 : full;
     }
     __syncthreads();
     bool hand = false;  // (FxArith) the location is left to the FP64 recursion
@@ -449,10 +449,12 @@ __global__ void __launch_bounds__(MBT, kScrThreads / MBT) select_mixed_kernel(co
       // multiple of 32 (all within Qpad; those past Qs only update state nobody reads), each
       // round's in two halves of whole warps
       const int Q32 = (Qs + 31) & ~31;
-      if constexpr (MBT == 512) {
+      // (two forms: the first alone spills in fixed point, the second alone runs the 256-thread
+      // float-float instance 4 % slower, n = 100 of 1000)
+      if constexpr (MBT == 512 || !A::kFixed) {
         const int per = sh_per;  // pairs of a round
         for (int base = 0, k = 0; base < Q32; base += per, k += NP) {
-          const int left = min(per, Q32 - base), dq = min(MBT, ((left >> 1) + 31) & ~31);
+          const int left = min(per, Q32 - base), dq = NP == 1 ? MBT : min(MBT, ((left >> 1) + 31) & ~31);
           if (tid < min(dq, left)) screen_pairs<A, MBT, NP, TM>(C, base + tid, b1, r1, b2, k, tid + dq < left ? dq : 0);
         }
       } else {
