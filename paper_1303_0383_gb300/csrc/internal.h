@@ -110,6 +110,7 @@ struct PredictArgs {
   const int32_t *nn = nullptr;
   int32_t M = 0;
   int64_t N = INT64_MAX;
+  int *queue = nullptr;  // a counter that is zero already, or nullptr: one in the workspace
   double *mean, *s2, *var;
   int8_t *status;
 };

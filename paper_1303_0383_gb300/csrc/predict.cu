@@ -284,10 +284,10 @@ int predict_fp64_launch(const PredictArgs &a, void *ws, size_t ws_bytes, cudaStr
   P.B = a.B;
   P.recip = a.recip; P.nn = a.nn; P.M = a.M; P.N = a.N;
   P.mean = a.mean; P.s2 = a.s2; P.var = a.var; P.status = a.status;
-  P.queue = reinterpret_cast<int *>(w);
+  P.queue = a.queue ? a.queue : reinterpret_cast<int *>(w);
   P.Ag = nullptr;
   P.group = 0;
-  cudaError_t e = cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
+  cudaError_t e = a.queue ? cudaSuccess : cudaMemsetAsync(P.queue, 0, sizeof(int), stream);
   if (e != cudaSuccess) return cuda_status(e);
   if (use_group(a.nmax)) {
     const GroupShape s = group_shape(a.T, a.nmax, di);

@@ -800,6 +800,7 @@ int mix_run(MixParams P, MixVariant v, const MixLayout &L, int G, char *w, size_
   pa.B.n_loc = P.n_out;  // adaptive designs: kernel (c) on each location's own size
   pa.recip = v.fixed;    // FP64: the recursion's own rounding, and no design where it fails
   pa.mean = P.mean; pa.s2 = P.s2; pa.var = P.var; pa.status = P.status;
+  pa.queue = reinterpret_cast<int *>(w + 192);  // (one of the counters: no launch between the two kernels)
   const int sp = predict_fp64_launch(pa, o, L.pred, stream);
   if (sp || !v.fixed) return sp;
   const size_t used = 512 + L.list;
