@@ -24,13 +24,14 @@ __device__ __forceinline__ int tri_row(int e) {
 }
 
 // a / l from q = rn(a r), r = rn(1 / l).  exact: also where the correction would leave the normal
-// range or meet an infinity (there it turns an infinite quotient into NaN), as a division.  With a
-// quotient within 2^-400 .. 2^400 and a pivot l = sqrt(v), 2^-537 .. 2^500, it does not.
+// range or meet an infinity (there it turns an infinite quotient into NaN), as a division.
 __device__ __forceinline__ double div_by_pivot(double a, double q, double l, double r, bool exact) {
-  const double c = fma(fma(-q, l, a), r, q);
-  if (exact && ((((unsigned)__double2hiint(q) >> 20) & 0x7ffu) - 623u) > 800u)
-    return a == 0.0 ? a : a / l;
-  return c;
+  if (exact) {
+    const unsigned ha = (unsigned)__double2hiint(a) & 0x7fffffffu, hq = (unsigned)__double2hiint(q) & 0x7fffffffu;
+    // both within 2^-960 .. 2^1023, or a = 0
+    if ((ha < (64u << 20) || hq < (64u << 20) || hq >= 0x7ff00000u) && (ha | (unsigned)__double2loint(a))) return a / l;
+  }
+  return fma(fma(-q, l, a), r, q);
 }
 
 // In-place Cholesky A = L L^T of the n x n lower triangle of A (row-major, leading
