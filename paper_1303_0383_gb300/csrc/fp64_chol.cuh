@@ -34,6 +34,13 @@ __device__ __forceinline__ double div_by_pivot(double a, double q, double l, dou
   return fma(fma(-q, l, a), r, q);
 }
 
+// Whether c, not zero, from div_by_pivot(a, q, l, r, false) is a / l: c within 2^-399 .. 2^399, so q
+// within 2^-400 .. 2^400.  With l = sqrt(v) within 2^-537 .. 2^512, a is then normal and the
+// residual a - q l, a multiple of 2^-1041, exact; a q beyond gives a c beyond (or NaN).
+__device__ __forceinline__ bool div_sure(double c) {
+  return (((unsigned)__double2hiint(c) >> 20 & 0x7ffu) - 624u) < 799u;
+}
+
 // In-place Cholesky A = L L^T of the n x n lower triangle of A (row-major, leading
 // dimension lda), carrying naug extra columns n .. n+naug-1 along so that they end as
 // L^{-1} b (forward substitution).  rl[k] receives 1 / l_kk.  Sets *fail (shared) on a
