@@ -67,8 +67,9 @@ extern "C" {
 typedef enum { LAGP_ALC = 0, LAGP_MSPE = 1, LAGP_NN = 2 } lagp_method;
 
 /* LAGP_FP64: every decision and every output in FP64, bit for bit those of the FP64
- * recursion (ALC: candidates are screened in 64-bit fixed point, at FP64's resolution, and
- * near-tied decisions taken by the recursion).
+ * recursion (ALC: candidates are screened in 64-bit fixed point, at FP64's resolution;
+ * near-tied decisions are taken in the recursion's arithmetic, and locations that fixed point
+ * does not resolve by the recursion itself).
  * LAGP_MIXED: the candidate screen (ALC or MSPE) runs in float-float (pairs of FP32,
  * about 48 significant bits) on the FP32 pipes; near-tied decisions, and MSPE scores whose
  * G or J is a cancellation beyond the screen's resolution, are re-scored in FP64.  The MSPE
